@@ -31,7 +31,10 @@ constexpr int oW1 = 0, oB1 = oW1 + kH * kIn, oW2 = oB1 + kH, oB2 = oW2 + kH * kH
               oB3 = oW3 + kH * kH, oW4 = oB3 + kH, oB4 = oW4 + kH, kNP = oB4 + 1;
 static_assert(kNP == GRTE_MLP_NPARAMS, "parameter count");
 
-// GELU (tanh form) and its derivative
+// GELU (tanh form) and its derivative.  (0.5 (1 + tanh u) as 1/(1 + exp(-2u)) from one
+// ex2.approx and one rcp.approx takes the inference kernel from 2.1x to 1.4x its
+// special-function bound and is no less accurate, but moves h by an ulp: every ~10^4th
+// activation then rounds to the other bfloat16 neighbour, and single predictions by 1e-2.)
 __device__ __forceinline__ float gelu(float z) {
   const float k = 0.7978845608028654f, c = 0.044715f;
   return 0.5f * z * (1.0f + tanhf(k * (z + c * z * z * z)));
@@ -94,19 +97,18 @@ struct MlpTile {   // shared memory of one block
   __nv_bfloat16 d3[kMlpSamples][kLd], d2[kMlpSamples][kLd], d1[kMlpSamples][kLd];
   float z1[kMlpSamples][kH], z2[kMlpSamples][kH], z3[kMlpSamples][kH];   // pre-activations, then deltas
   float d4[kMlpSamples], err2[kMlpSamples];
-  float g[kNP];                             // block gradient (MODE 1)
+  float g[kNP];                             // block gradient
 };
 
-// Forward and (MODE 1) backward of 64 samples per block: MODE 0 writes predictions;
-// MODE 1 writes the block's gradient (sum over its samples of d(loss)/d(param), loss =
-// mean of squared standardised errors, `scale` = 1/n) to part[blockIdx.x][kNP] and its
-// summed squared error to loss_part.  Samples past n enter with zero inputs and zero
-// output gradient.
-template <int MODE>
-__global__ void __launch_bounds__(kMlpThreads) k_mlp(const __nv_bfloat16* __restrict__ wts, const float* __restrict__ X,
-                                                     const float* __restrict__ Y, int64_t n, const float* __restrict__ norm,
-                                                     float* __restrict__ out, float* __restrict__ part,
-                                                     float* __restrict__ loss_part, float scale) {
+// Forward and backward of 64 samples per block: writes the block's gradient (sum over its
+// samples of d(loss)/d(param), loss = mean of squared standardised errors, `scale` = 1/n) to
+// part[blockIdx.x][kNP] and its summed squared error to loss_part.  Samples past n enter with
+// zero inputs and zero output gradient.
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(const __nv_bfloat16* __restrict__ wts,
+                                                          const float* __restrict__ X, const float* __restrict__ Y,
+                                                          int64_t n, const float* __restrict__ norm,
+                                                          float* __restrict__ part, float* __restrict__ loss_part,
+                                                          float scale) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpTile& S = *reinterpret_cast<MlpTile*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const __nv_bfloat16* __rest
   const int64_t s0 = (int64_t)blockIdx.x * kMlpSamples;
   for (int i = tid; i < kNP; i += kMlpThreads) {
     S.w[i] = wts[i];
-    if (MODE == 1) S.g[i] = 0.0f;
+    S.g[i] = 0.0f;
   }
   for (int i = tid; i < kH * 16; i += kMlpThreads) {
     const int j = i / 16, k = i % 16;
@@ -183,14 +185,6 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const __nv_bfloat16* __rest
     o[hh] += __shfl_xor_sync(0xffffffffu, o[hh], 1);
     o[hh] += __shfl_xor_sync(0xffffffffu, o[hh], 2);
     o[hh] += __bfloat162float(W[oB4]);
-  }
-  if (MODE == 0) {
-    if (q == 0)
-      for (int hh = 0; hh < 2; ++hh) {
-        const int64_t s = s0 + r0 + g8 + hh * 8;
-        if (s < n) out[s] = o[hh] * norm[2 * kIn + 1] + norm[2 * kIn];   // un-standardised prediction
-      }
-    return;
   }
   // ---- backward
   float d4r[2];
@@ -293,6 +287,154 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const __nv_bfloat16* __rest
   }
 }
 
+// ----------------------------------------------------------------------------- inference
+// The network on n raw feature rows.  A warp takes TILES x 16 samples at a time and carries
+// them through all layers in registers: an accumulator of m16n8k16 holds exactly the elements
+// that the next layer's A fragment wants in the same lane (columns 2q, 2q+1 of rows g, g+8),
+// so no activation touches shared memory and warps never wait for each other.  The weights
+// are laid out once per block as B fragments (8 bytes per lane, one conflict-free LDS.64 per
+// fragment, used for TILES products); blocks stay and stride over the samples.
+// Bound: instruction issue of the 192 tanhf per sample (the products are 6% of the time and
+// the special-function unit's share is 83 us).  2^20 samples: 288 us (3.6e9 samples/s, 63
+// TFLOP/s of products), against 1013 us with one 64-sample tile per block, whose weights were
+// loaded again for every tile and whose activations went through shared memory.
+// TILES: two tiles per warp read each fragment half as often; one spreads small n over more
+// warps (kInferWide below).
+constexpr int kInferThreads = 128;
+struct InferSmem {
+  uint2 b1[8][32];            // layer 1, K = 16 (6 inputs, rest 0): [n-tile][lane]
+  uint2 b2[8][4][32], b3[8][4][32];   // layers 2, 3: [n-tile][k-tile][lane]
+  float c1[kH], c2[kH], c3[kH], w4[kH];
+  float mean[8], std[8];
+  float c4, ym, ys;
+};
+
+__device__ __forceinline__ uint32_t pack_f2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+template <int TILES>
+__global__ void __launch_bounds__(kInferThreads, 4) k_mlp_infer(const __nv_bfloat16* __restrict__ wts,
+                                                               const float* __restrict__ X, int64_t n,
+                                                               const float* __restrict__ norm,
+                                                               float* __restrict__ out) {
+  __shared__ InferSmem S;
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int g = lane >> 2, q = lane & 3;
+  {
+    // each warp lays out fragments for its own lane positions
+    auto pair = [&](int off) { return *reinterpret_cast<const uint32_t*>(wts + off); };   // off is even
+    for (int f = wp; f < 8; f += kInferThreads / 32)
+      S.b1[f][lane] = make_uint2(q < kIn / 2 ? pair(oW1 + (f * 8 + g) * kIn + 2 * q) : 0u, 0u);
+    for (int f = wp; f < 32; f += kInferThreads / 32) {
+      const int o = (((f >> 2) * 8 + g) * kH) + (f & 3) * 16 + 2 * q;
+      S.b2[f >> 2][f & 3][lane] = make_uint2(pair(oW2 + o), pair(oW2 + o + 8));
+      S.b3[f >> 2][f & 3][lane] = make_uint2(pair(oW3 + o), pair(oW3 + o + 8));
+    }
+    if (tid < kH) {
+      S.c1[tid] = __bfloat162float(wts[oB1 + tid]);
+      S.c2[tid] = __bfloat162float(wts[oB2 + tid]);
+      S.c3[tid] = __bfloat162float(wts[oB3 + tid]);
+      S.w4[tid] = __bfloat162float(wts[oW4 + tid]);
+    } else if (tid < kH + kIn) {
+      S.mean[tid - kH] = norm[tid - kH];
+      S.std[tid - kH] = norm[kIn + tid - kH];
+    } else if (tid == kH + 8) {
+      S.c4 = __bfloat162float(wts[oB4]);
+      S.ym = norm[2 * kIn];
+      S.ys = norm[2 * kIn + 1];
+    }
+  }
+  __syncthreads();
+  constexpr int kRows = 16 * TILES;
+  const int64_t nwarp = (int64_t)gridDim.x * (kInferThreads / 32);
+  for (int64_t s0 = ((int64_t)blockIdx.x * (kInferThreads / 32) + wp) * kRows; s0 < n; s0 += nwarp * kRows) {
+    // standardised inputs as the A fragment of layer 1 (columns 8..15 are 0)
+    uint32_t x[TILES][2];
+#pragma unroll
+    for (int t = 0; t < TILES; ++t)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        const int64_t s = s0 + t * 16 + hh * 8 + g;
+        float v0 = 0.0f, v1 = 0.0f;
+        if (q < kIn / 2 && s < n) {
+          v0 = (X[s * kIn + 2 * q] - S.mean[2 * q]) / S.std[2 * q];
+          v1 = (X[s * kIn + 2 * q + 1] - S.mean[2 * q + 1]) / S.std[2 * q + 1];
+        }
+        x[t][hh] = pack_f2(v0, v1);
+      }
+    uint32_t h1[TILES][4][4], h2[TILES][4][4];   // A fragments of layers 2 and 3
+    float o[TILES][2];
+#pragma unroll
+    for (int t = 0; t < TILES; ++t) o[t][0] = o[t][1] = 0.0f;
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+      const float2 bias = *reinterpret_cast<const float2*>(&S.c1[nt * 8 + 2 * q]);
+      const uint2 b = S.b1[nt][lane];
+#pragma unroll
+      for (int t = 0; t < TILES; ++t) {
+        float c[4] = {bias.x, bias.y, bias.x, bias.y};
+        const uint32_t a[4] = {x[t][0], x[t][1], 0u, 0u}, bb[2] = {b.x, b.y};
+        mma16816(c, a, bb);
+        h1[t][nt >> 1][(nt & 1) * 2] = pack_f2(gelu(c[0]), gelu(c[1]));
+        h1[t][nt >> 1][(nt & 1) * 2 + 1] = pack_f2(gelu(c[2]), gelu(c[3]));
+      }
+    }
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+      const float2 bias = *reinterpret_cast<const float2*>(&S.c2[nt * 8 + 2 * q]);
+      float c[TILES][4];
+#pragma unroll
+      for (int t = 0; t < TILES; ++t) c[t][0] = c[t][2] = bias.x, c[t][1] = c[t][3] = bias.y;
+#pragma unroll
+      for (int kt = 0; kt < 4; ++kt) {
+        const uint2 b = S.b2[nt][kt][lane];
+        const uint32_t bb[2] = {b.x, b.y};
+#pragma unroll
+        for (int t = 0; t < TILES; ++t) mma16816(c[t], h1[t][kt], bb);
+      }
+#pragma unroll
+      for (int t = 0; t < TILES; ++t) {
+        h2[t][nt >> 1][(nt & 1) * 2] = pack_f2(gelu(c[t][0]), gelu(c[t][1]));
+        h2[t][nt >> 1][(nt & 1) * 2 + 1] = pack_f2(gelu(c[t][2]), gelu(c[t][3]));
+      }
+    }
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+      const float2 bias = *reinterpret_cast<const float2*>(&S.c3[nt * 8 + 2 * q]);
+      const float2 w4 = *reinterpret_cast<const float2*>(&S.w4[nt * 8 + 2 * q]);
+      float c[TILES][4];
+#pragma unroll
+      for (int t = 0; t < TILES; ++t) c[t][0] = c[t][2] = bias.x, c[t][1] = c[t][3] = bias.y;
+#pragma unroll
+      for (int kt = 0; kt < 4; ++kt) {
+        const uint2 b = S.b3[nt][kt][lane];
+        const uint32_t bb[2] = {b.x, b.y};
+#pragma unroll
+        for (int t = 0; t < TILES; ++t) mma16816(c[t], h2[t][kt], bb);
+      }
+#pragma unroll
+      for (int t = 0; t < TILES; ++t)
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          o[t][hh] = fmaf(w4.x, gelu(c[t][2 * hh]), o[t][hh]);
+          o[t][hh] = fmaf(w4.y, gelu(c[t][2 * hh + 1]), o[t][hh]);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < TILES; ++t)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        float v = o[t][hh];
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        const int64_t s = s0 + t * 16 + hh * 8 + g;
+        if (q == 0 && s < n) out[s] = (v + S.c4) * S.ys + S.ym;   // un-standardised prediction
+      }
+  }
+}
+
 // Sum the per-block partial gradients (fixed order) into grad.
 __global__ void k_mlp_reduce(const float* __restrict__ part, int nblk, float* __restrict__ grad) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -323,7 +465,19 @@ __global__ void k_to_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict
   if (i < kNP) wb[i] = __float2bfloat16(p[i]);
 }
 
-size_t mlp_smem_bytes(int) { return sizeof(MlpTile); }
+// Two tiles per warp from the n at which one tile would give every SM four blocks (below
+// that, more warps matter more than fragment reads).
+constexpr int64_t kInferWide = 16 * (kInferThreads / 32) * 152 * 4;
+
+static cudaError_t infer_launch(const __nv_bfloat16* wb, const float* norm, const float* X, int64_t n, float* y,
+                                cudaStream_t stream) {
+  const bool wide = n >= kInferWide;
+  const int64_t per = (int64_t)(wide ? 32 : 16) * (kInferThreads / 32);
+  const int nb = (int)std::min<int64_t>((n + per - 1) / per, 152 * 4);
+  if (wide) k_mlp_infer<2><<<nb, kInferThreads, 0, stream>>>(wb, X, n, norm, y);
+  else k_mlp_infer<1><<<nb, kInferThreads, 0, stream>>>(wb, X, n, norm, y);
+  return cudaGetLastError();
+}
 
 }  // namespace grte
 
@@ -354,10 +508,7 @@ static grte_status mfail(grte_mlp_t h, grte_status s, const std::string& m) {
 namespace grte {
 cudaError_t mlp_guess_launch(grte_mlp_t h, const float* feat, int64_t n, float* y, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
-  const int nb = (int)((n + kMlpSamples - 1) / kMlpSamples);
-  k_mlp<0><<<nb, kMlpThreads, mlp_smem_bytes(0), stream>>>(h->wb, feat, nullptr, n, h->norm, y, nullptr, nullptr,
-                                                            0.0f);
-  return cudaGetLastError();
+  return infer_launch(h->wb, h->norm, feat, n, y, stream);
 }
 }  // namespace grte
 
@@ -398,8 +549,7 @@ grte_status grte_mlp_create(uint64_t seed, grte_mlp_t* out) {
   h->hnorm[2 * kIn] = 0.0f;
   h->hnorm[2 * kIn + 1] = 1.0f;
   MCK(cudaMemcpy(h->norm, h->hnorm, sizeof(h->hnorm), cudaMemcpyHostToDevice));
-  MCK(cudaFuncSetAttribute(k_mlp<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes(0)));
-  MCK(cudaFuncSetAttribute(k_mlp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes(1)));
+  MCK(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile)));
   return GRTE_OK;
 }
 
@@ -456,9 +606,7 @@ grte_status grte_mlp_forward(grte_mlp_t h, const float* X, int64_t n, float* y) 
   MCK(cudaMalloc(&dX, sizeof(float) * n * kIn));
   MCK(cudaMalloc(&dY, sizeof(float) * n));
   MCK(cudaMemcpy(dX, X, sizeof(float) * n * kIn, cudaMemcpyHostToDevice));
-  const int nb = (int)((n + kMlpSamples - 1) / kMlpSamples);
-  k_mlp<0><<<nb, kMlpThreads, mlp_smem_bytes(0)>>>(h->wb, dX, nullptr, n, h->norm, dY, nullptr, nullptr, 0.0f);
-  MCK(cudaGetLastError());
+  MCK(infer_launch(h->wb, h->norm, dX, n, dY, nullptr));
   MCK(cudaMemcpy(y, dY, sizeof(float) * n, cudaMemcpyDeviceToHost));
   cudaFree(dX);
   cudaFree(dY);
@@ -468,8 +616,7 @@ grte_status grte_mlp_forward(grte_mlp_t h, const float* X, int64_t n, float* y) 
 static grte_status grad_batch(grte_mlp_t h, const float* dX, const float* dY, int64_t n, float* dpart,
                               float* dlpart, float* loss) {
   const int nb = (int)((n + kMlpSamples - 1) / kMlpSamples);
-  k_mlp<1><<<nb, kMlpThreads, mlp_smem_bytes(1)>>>(h->wb, dX, dY, n, h->norm, nullptr, dpart, dlpart,
-                                                    1.0f / (float)n);
+  k_mlp_grad<<<nb, kMlpThreads, sizeof(MlpTile)>>>(h->wb, dX, dY, n, h->norm, dpart, dlpart, 1.0f / (float)n);
   MCK(cudaGetLastError());
   k_mlp_reduce<<<(kNP + 255) / 256, 256>>>(dpart, nb, h->g);
   MCK(cudaGetLastError());
