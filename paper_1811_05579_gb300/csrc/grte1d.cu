@@ -1425,6 +1425,9 @@ struct grte_ctx {
   bool fused = false;
   int* d_finst = nullptr;
   int fcnt[5] = {0, 0, 0, 0, 0}, foff[5] = {0, 0, 0, 0, 0};
+  // handles with several cluster sizes: side streams of the smaller ones (fused_solves)
+  cudaStream_t fstream[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t fev_fork = nullptr, fev_join[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaEvent_t ev_state = nullptr;   // grte_get_T_device: the caller's stream waits on it
 };
 
@@ -1658,11 +1661,42 @@ static cudaError_t fused_schedulable(int Qc, int m, bool* ok) {
   return e;
 }
 
-static cudaError_t fused_launch(grte_ctx* h, int c) {
+static cudaError_t fused_launch(grte_ctx* h, int c, cudaStream_t st) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  fused_config(cfg, at, 1 << c, h->fcnt[c], h->D.m, h->stream);
+  fused_config(cfg, at, 1 << c, h->fcnt[c], h->D.m, st);
   return cudaLaunchKernelEx(&cfg, k_pred_fused, h->D, (const int*)(h->d_finst + h->foff[c]));
+}
+
+// The prediction solves of all instances.  The launches of different cluster sizes have no
+// data in common (each instance belongs to one), so the smaller sizes run on side streams
+// beside the largest, between a fork and a join on the handle's stream: one launch rarely
+// fills the chip (at most seven 16-CTA clusters fit, a one-CTA class has one CTA per
+// instance), and in turn each waits for the slowest solve of the one before.  The largest
+// size is launched first: its clusters need the most free SMs at once, and its solves take
+// longest.  64 uneven instances: 2.04 ms of solves per step in turn, 1.10 side by side.
+// With per-kernel timing on they run in turn, so that each event pair times its launch alone.
+static cudaError_t fused_solves(grte_ctx* h) {
+  cudaStream_t st = h->stream;
+  cudaError_t e = cudaSuccess;
+  if (!h->fev_fork || h->prof_mask != 0) {
+    for (int c = 4; c >= 0 && e == cudaSuccess; --c)
+      if (h->fcnt[c]) LAUNCH(GRTE_K_PRED_SOLVE, e = fused_launch(h, c, st));
+    return e;
+  }
+  e = cudaEventRecord(h->fev_fork, st);
+  int side = -1;   // the largest size runs on the handle's stream
+  for (int c = 4; c >= 0 && e == cudaSuccess; --c) {
+    if (!h->fcnt[c]) continue;
+    cudaStream_t s = side < 0 ? st : h->fstream[side];
+    if (side >= 0) e = cudaStreamWaitEvent(s, h->fev_fork, 0);
+    if (e == cudaSuccess) e = fused_launch(h, c, s);
+    ++h->launches;
+    if (side >= 0 && e == cudaSuccess) e = cudaEventRecord(h->fev_join[side], s);
+    ++side;
+  }
+  for (int i = 0; i < side && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(st, h->fev_join[i], 0);
+  return e;
 }
 
 // Krylov iterations and restart cycles of the fused solve, accumulated over graph replays.
@@ -1780,6 +1814,9 @@ void grte_destroy(grte_t h) {
   if (h->h_flags) cudaFreeHost(h->h_flags);
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   if (h->ev_state) cudaEventDestroy(h->ev_state);
+  if (h->fev_fork) cudaEventDestroy(h->fev_fork);
+  for (cudaEvent_t e : h->fev_join) if (e) cudaEventDestroy(e);
+  for (cudaStream_t s : h->fstream) if (s) cudaStreamDestroy(s);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
@@ -2036,6 +2073,12 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
       CK(cudaMemcpy(h->d_finst, order.data(), sizeof(int) * n_inst, cudaMemcpyHostToDevice));
       CK(cudaMemcpy(h->d_inst, h->inst.data(), sizeof(Inst) * n_inst, cudaMemcpyHostToDevice));
       h->fused = true;
+      const int nsize = (int)std::count_if(h->fcnt, h->fcnt + 5, [](int n) { return n > 0; });
+      for (int i = 0; i + 1 < nsize; ++i) {
+        CK(cudaStreamCreateWithFlags(&h->fstream[i], cudaStreamNonBlocking));
+        CK(cudaEventCreateWithFlags(&h->fev_join[i], cudaEventDisableTiming));
+      }
+      if (nsize > 1) CK(cudaEventCreateWithFlags(&h->fev_fork, cudaEventDisableTiming));
     }
   }
   return GRTE_OK;
@@ -2184,12 +2227,7 @@ static grte_status step_fused(grte_t h, bool allow_tune) {
   LAUNCH(GRTE_K_CELL_COEF, k_cell_coef<<<G.cgrid, G.cb, 0, st>>>(D, G.ni, h->d_cell_start, G.nc, 0));
   LAUNCH(GRTE_K_RHO, k_rho<R><<<G.cgrid, G.cb, 0, st>>>(D, G.ni, h->d_cell_start, G.nc, D.rho_n));
   CK(cudaMemcpyAsync(D.gx, D.rho_n, sizeof(double) * G.nc, cudaMemcpyDeviceToDevice, st));
-  for (int c = 0; c < 5; ++c) {
-    if (!h->fcnt[c]) continue;
-    cudaError_t e = cudaSuccess;
-    LAUNCH(GRTE_K_PRED_SOLVE, e = fused_launch(h, c));
-    CK(e);
-  }
+  CK(fused_solves(h));
   if (h->nt == 0) {
     if (!allow_tune) return fail(h, GRTE_ESTATE, "line solves not tuned");
     // the correction's line solves are tuned on this step's per-cell parts
