@@ -39,6 +39,7 @@ struct NvtxRange {
 };
 }  // namespace
 #include "mlp.cuh"
+#include "stateio.cuh"
 #include "tridiag.cuh"
 
 namespace grte {
@@ -2084,35 +2085,53 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   return GRTE_OK;
 }
 
+}  // extern "C"
+
+// Device scratch for one instance's state in the host's layout: the factor storage of its
+// lines, which every step factors anew (5 values of at least 4 bytes per line element, so
+// room for two binary64 arrays of N M values, or one of (N + 1) M).
+static double* io_stage(grte_t h, const Inst& I) {
+  const size_t es = h->opt.precision == GRTE_MIXED ? 4 : 8;
+  const uintptr_t p = (uintptr_t)h->D.F + es * (size_t)h->lines[I.line_off].f_off;
+  return (double*)((p + 7) & ~(uintptr_t)7);
+}
+
+// The instance's device lines from E and O in the host's layout (NULL: equilibrium, 0).  E is
+// stored as its deviation Eh = E - a c U.
+template <typename R>
+static grte_status lines_in(grte_t h, const Inst& I, const double* E, const double* O) {
+  Dev& D = h->D;
+  const int64_t N = I.N;
+  R *Eh = (R*)D.Eh + I.elem_off, *On = (R*)D.O + I.nelem_off;
+  if (!E) {
+    CK(cudaMemsetAsync(Eh, 0, sizeof(R) * N * I.M, h->stream));
+    CK(cudaMemsetAsync(On, 0, sizeof(R) * (N + 1) * I.M, h->stream));
+    return GRTE_OK;
+  }
+  double* st = io_stage(h, I);
+  CK(cudaMemcpyAsync(st, E, sizeof(double) * N * I.M, cudaMemcpyHostToDevice, h->stream));
+  k_lines_in<R><<<io_grid(N, I.M), io_block(), 0, h->stream>>>(st, Eh, N, I.M, D.U + I.cell_off, I.a * I.c);
+  CK(cudaMemcpyAsync(st, O, sizeof(double) * (N + 1) * I.M, cudaMemcpyHostToDevice, h->stream));
+  k_lines_in<R><<<io_grid(N + 1, I.M), io_block(), 0, h->stream>>>(st, On, N + 1, I.M, nullptr, 0.0);
+  CK(cudaGetLastError());
+  return GRTE_OK;
+}
+
+extern "C" {
+
 grte_status grte_set_state(grte_t h, int inst, const double* T, const double* E, const double* O) {
   if (!h) return GRTE_EINVAL;
   if (inst < 0 || inst >= h->n_inst || !T) return fail(h, GRTE_EINVAL, "bad instance or T NULL");
   if ((E == nullptr) != (O == nullptr)) return fail(h, GRTE_EINVAL, "E and O must both be given or both NULL");
   const Inst& I = h->inst[inst];
-  const int64_t N = I.N, M = I.M;
-  std::vector<double> hE(N * M), hO((N + 1) * M), hU(N);
-  for (int64_t j = 0; j < N; ++j) {
+  for (int64_t j = 0; j < I.N; ++j)
     if (!(T[j] >= 0.0) || !std::isfinite(T[j])) return fail(h, GRTE_EINVAL, "T must be finite and >= 0");
-    hU[j] = (T[j] * T[j]) * (T[j] * T[j]);
-  }
-  // device layout: line-major, E stored as its deviation Eh = E - a c U
-  for (int64_t k = 0; k < M; ++k) {
-    for (int64_t j = 0; j < N; ++j) hE[k * N + j] = E ? E[j * M + k] - I.a * I.c * hU[j] : 0.0;
-    for (int64_t i = 0; i <= N; ++i) hO[k * (N + 1) + i] = O ? O[i * M + k] : 0.0;
-  }
   Dev& D = h->D;
-  CK(cudaMemcpyAsync(D.T + I.cell_off, T, sizeof(double) * N, cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(D.U + I.cell_off, hU.data(), sizeof(double) * N, cudaMemcpyHostToDevice, h->stream));
-  if (h->opt.precision == GRTE_MIXED) {
-    std::vector<float> fE(hE.begin(), hE.end()), fO(hO.begin(), hO.end());
-    CK(cudaMemcpyAsync((float*)D.Eh + I.elem_off, fE.data(), sizeof(float) * N * M, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync((float*)D.O + I.nelem_off, fO.data(), sizeof(float) * (N + 1) * M, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-  } else {
-    CK(cudaMemcpyAsync((double*)D.Eh + I.elem_off, hE.data(), sizeof(double) * N * M, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync((double*)D.O + I.nelem_off, hO.data(), sizeof(double) * (N + 1) * M, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-  }
+  CK(cudaMemcpyAsync(D.T + I.cell_off, T, sizeof(double) * I.N, cudaMemcpyHostToDevice, h->stream));
+  k_fourth_power<<<(unsigned)((I.N + 255) / 256), 256, 0, h->stream>>>(D.T + I.cell_off, D.U + I.cell_off, I.N);
+  const grte_status s = h->opt.precision == GRTE_MIXED ? lines_in<float>(h, I, E, O) : lines_in<double>(h, I, E, O);
+  if (s != GRTE_OK) return s;
+  CK(cudaStreamSynchronize(h->stream));
   h->inst_set[inst] = 1;
   h->state_set = std::all_of(h->inst_set.begin(), h->inst_set.end(), [](char c) { return c != 0; });
   return GRTE_OK;
@@ -2585,11 +2604,10 @@ grte_status grte_step(grte_t h, int64_t nsteps) {
 }
 
 static grte_status device_status(grte_t h) {
-  std::vector<int> s(h->n_inst);
+  CK(cudaMemcpyAsync(h->h_flags, h->D.status, sizeof(int) * h->n_inst, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  CK(cudaMemcpy(s.data(), h->D.status, sizeof(int) * h->n_inst, cudaMemcpyDeviceToHost));
   int64_t all = 0;
-  for (int v : s) all |= v;
+  for (int i = 0; i < h->n_inst; ++i) all |= h->h_flags[i];
   h->stats.status_flags = all;
   for (int code : {GRTE_ENAN, GRTE_ENONCONV, GRTE_ENEGATIVE, GRTE_ETIMEOUT})
     if (all & (1 << code)) return fail(h, (grte_status)code, "device reported status " + std::to_string(code));
@@ -2609,8 +2627,7 @@ static grte_status get_cells(grte_t h, int inst, const double* src, double* out,
   if (inst < 0 || inst >= h->n_inst || !out) return fail(h, GRTE_EINVAL, "bad instance or NULL output");
   const Inst& I = h->inst[inst];
   if (len != (size_t)I.N) return fail(h, GRTE_EINVAL, "len must equal nx");
-  CK(cudaStreamSynchronize(h->stream));
-  CK(cudaMemcpy(out, src + I.cell_off, sizeof(double) * I.N, cudaMemcpyDeviceToHost));
+  CK(cudaMemcpyAsync(out, src + I.cell_off, sizeof(double) * I.N, cudaMemcpyDeviceToHost, h->stream));
   return device_status(h);
 }
 
@@ -2627,44 +2644,79 @@ grte_status grte_get_stage(grte_t h, int inst, int which, double* out, size_t le
   return get_cells(h, inst, src, out, len);
 }
 
-// Copy n bulk elements from device offset `off` (in elements) of `base` into doubles.
-static grte_status copy_bulk(grte_t h, const void* base, int64_t off, int64_t n, double* out) {
-  CK(cudaStreamSynchronize(h->stream));
-  if (h->opt.precision == GRTE_MIXED) {
-    std::vector<float> t(n);
-    CK(cudaMemcpy(t.data(), (const float*)base + off, sizeof(float) * n, cudaMemcpyDeviceToHost));
-    for (int64_t i = 0; i < n; ++i) out[i] = t[i];
-  } else {
-    CK(cudaMemcpy(out, (const double*)base + off, sizeof(double) * n, cudaMemcpyDeviceToHost));
+}  // extern "C"
+
+// E (even) or O of an instance in the host's layout, on the device scratch.
+template <typename R>
+static double* lines_out(grte_t h, const Inst& I, bool even) {
+  const Dev& D = h->D;
+  double* st = io_stage(h, I);
+  const int64_t rows = even ? I.N : I.N + 1;
+  const R* src = even ? (const R*)D.Eh + I.elem_off : (const R*)D.O + I.nelem_off;
+  k_lines_out<R><<<io_grid(rows, I.M), io_block(), 0, h->stream>>>(src, st, rows, I.M,
+                                                                   even ? D.U + I.cell_off : nullptr, I.a * I.c);
+  return st;
+}
+
+// rho = sum_k w_k E_k per cell, fixed angle order
+template <typename R>
+__global__ void k_moment_out(Dev D, Inst I, double* __restrict__ rho) {
+  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (j >= I.N) return;
+  const R* Eh = (const R*)D.Eh + I.elem_off;
+  const double acU = I.a * I.c * D.U[I.cell_off + j];
+  double acc = 0.0;
+  for (int k = 0; k < I.M; ++k) acc += D.w[I.ang_off + k] * (acU + (double)Eh[(int64_t)k * I.N + j]);
+  rho[j] = acc;
+}
+
+// Cell-centre intensities I(+-v_k) = E +- eps (O_j + O_{j+1})/2 in the host's layout
+// (tiles as in k_lines_out)
+template <typename R>
+__global__ void k_intensity_out(Dev D, Inst I, double* __restrict__ Ipos, double* __restrict__ Ineg) {
+  __shared__ double te[kIoTile][kIoTile + 1], to[kIoTile][kIoTile + 1];
+  const int64_t j0 = (int64_t)blockIdx.x * kIoTile;
+  const int k0 = blockIdx.y * kIoTile;
+  const int64_t j = j0 + threadIdx.x;
+  if (j < I.N) {
+    const double acU = I.a * I.c * D.U[I.cell_off + j];
+    for (int r = threadIdx.y; r < kIoTile && k0 + r < I.M; r += kIoRows) {
+      const int k = k0 + r;
+      const R* On = (const R*)D.O + I.nelem_off + (int64_t)k * (I.N + 1);
+      te[r][threadIdx.x] = acU + (double)((const R*)D.Eh)[I.elem_off + (int64_t)k * I.N + j];
+      to[r][threadIdx.x] = 0.5 * ((double)On[j] + (double)On[j + 1]);
+    }
   }
-  return GRTE_OK;
+  __syncthreads();
+  const int k = k0 + threadIdx.x;
+  if (k >= I.M) return;
+  for (int r = threadIdx.y; r < kIoTile; r += kIoRows) {
+    const int64_t jj = j0 + r;
+    if (jj >= I.N) continue;
+    Ipos[jj * I.M + k] = te[threadIdx.x][r] + I.eps * to[threadIdx.x][r];
+    Ineg[jj * I.M + k] = te[threadIdx.x][r] - I.eps * to[threadIdx.x][r];
+  }
+}
+
+extern "C" {
+
+static grte_status get_lines(grte_t h, int inst, bool even, double* out, size_t len) {
+  if (inst < 0 || inst >= h->n_inst || !out) return fail(h, GRTE_EINVAL, "bad instance or NULL output");
+  const Inst& I = h->inst[inst];
+  const size_t need = (size_t)(even ? I.N : I.N + 1) * I.M;
+  if (len != need) return fail(h, GRTE_EINVAL, even ? "len must equal nx*M" : "len must equal (nx+1)*M");
+  const double* st = h->opt.precision == GRTE_MIXED ? lines_out<float>(h, I, even) : lines_out<double>(h, I, even);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(out, st, sizeof(double) * need, cudaMemcpyDeviceToHost, h->stream));
+  return device_status(h);
 }
 
 grte_status grte_get_E(grte_t h, int inst, double* E, size_t len) {
-  if (!h) return GRTE_EINVAL;
-  if (inst < 0 || inst >= h->n_inst || !E) return fail(h, GRTE_EINVAL, "bad instance or NULL output");
-  const Inst& I = h->inst[inst];
-  if (len != (size_t)I.N * I.M) return fail(h, GRTE_EINVAL, "len must equal nx*M");
-  std::vector<double> t((size_t)I.N * I.M), U(I.N);
-  grte_status s = copy_bulk(h, h->D.Eh, I.elem_off, (int64_t)t.size(), t.data());
-  if (s != GRTE_OK) return s;
-  CK(cudaMemcpy(U.data(), h->D.U + I.cell_off, sizeof(double) * I.N, cudaMemcpyDeviceToHost));
-  for (int64_t k = 0; k < I.M; ++k)
-    for (int64_t j = 0; j < I.N; ++j) E[j * I.M + k] = I.a * I.c * U[j] + t[k * I.N + j];
-  return device_status(h);
+  return h ? get_lines(h, inst, true, E, len) : GRTE_EINVAL;
 }
 
 grte_status grte_get_O(grte_t h, int inst, double* O, size_t len) {
-  if (!h) return GRTE_EINVAL;
-  if (inst < 0 || inst >= h->n_inst || !O) return fail(h, GRTE_EINVAL, "bad instance or NULL output");
-  const Inst& I = h->inst[inst];
-  if (len != (size_t)(I.N + 1) * I.M) return fail(h, GRTE_EINVAL, "len must equal (nx+1)*M");
-  std::vector<double> t((size_t)(I.N + 1) * I.M);
-  grte_status s = copy_bulk(h, h->D.O, I.nelem_off, (int64_t)t.size(), t.data());
-  if (s != GRTE_OK) return s;
-  for (int64_t k = 0; k < I.M; ++k)
-    for (int64_t i = 0; i <= I.N; ++i) O[i * I.M + k] = t[k * (I.N + 1) + i];
-  return device_status(h);
+  return h ? get_lines(h, inst, false, O, len) : GRTE_EINVAL;
 }
 
 grte_status grte_get_rho(grte_t h, int inst, double* rho, size_t len) {
@@ -2672,34 +2724,30 @@ grte_status grte_get_rho(grte_t h, int inst, double* rho, size_t len) {
   if (inst < 0 || inst >= h->n_inst || !rho) return fail(h, GRTE_EINVAL, "bad instance or NULL output");
   const Inst& I = h->inst[inst];
   if (len != (size_t)I.N) return fail(h, GRTE_EINVAL, "len must equal nx");
-  std::vector<double> E((size_t)I.N * I.M);
-  grte_status s = grte_get_E(h, inst, E.data(), E.size());
-  if (s != GRTE_OK && s != GRTE_ENEGATIVE) return s;
-  for (int64_t j = 0; j < I.N; ++j) {
-    double acc = 0.0;
-    for (int k = 0; k < I.M; ++k) acc += h->hw[I.ang_off + k] * E[j * I.M + k];
-    rho[j] = acc;
-  }
-  return s;
+  double* st = io_stage(h, I);
+  const unsigned nb = (unsigned)((I.N + 255) / 256);
+  if (h->opt.precision == GRTE_MIXED) k_moment_out<float><<<nb, 256, 0, h->stream>>>(h->D, I, st);
+  else k_moment_out<double><<<nb, 256, 0, h->stream>>>(h->D, I, st);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(rho, st, sizeof(double) * I.N, cudaMemcpyDeviceToHost, h->stream));
+  return device_status(h);
 }
 
 grte_status grte_get_I(grte_t h, int inst, double* Ipos, double* Ineg, size_t len) {
   if (!h) return GRTE_EINVAL;
   if (inst < 0 || inst >= h->n_inst || !Ipos || !Ineg) return fail(h, GRTE_EINVAL, "bad instance or NULL output");
   const Inst& I = h->inst[inst];
-  if (len != (size_t)I.N * I.M) return fail(h, GRTE_EINVAL, "len must equal nx*M");
-  std::vector<double> E((size_t)I.N * I.M), O((size_t)(I.N + 1) * I.M);
-  grte_status s = grte_get_E(h, inst, E.data(), E.size());
-  if (s != GRTE_OK && s != GRTE_ENEGATIVE) return s;
-  s = grte_get_O(h, inst, O.data(), O.size());
-  if (s != GRTE_OK && s != GRTE_ENEGATIVE) return s;
-  for (int64_t j = 0; j < I.N; ++j)
-    for (int k = 0; k < I.M; ++k) {
-      const double oc = 0.5 * (O[j * I.M + k] + O[(j + 1) * I.M + k]);
-      Ipos[j * I.M + k] = E[j * I.M + k] + I.eps * oc;
-      Ineg[j * I.M + k] = E[j * I.M + k] - I.eps * oc;
-    }
-  return s;
+  const int64_t n = (int64_t)I.N * I.M;
+  if (len != (size_t)n) return fail(h, GRTE_EINVAL, "len must equal nx*M");
+  double* st = io_stage(h, I);
+  if (h->opt.precision == GRTE_MIXED)
+    k_intensity_out<float><<<io_grid(I.N, I.M), io_block(), 0, h->stream>>>(h->D, I, st, st + n);
+  else
+    k_intensity_out<double><<<io_grid(I.N, I.M), io_block(), 0, h->stream>>>(h->D, I, st, st + n);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(Ipos, st, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaMemcpyAsync(Ineg, st + n, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
+  return device_status(h);
 }
 
 // Checkpoint blob: a header, the per-instance sizes, the energy sums and the raw device

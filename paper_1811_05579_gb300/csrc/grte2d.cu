@@ -34,6 +34,7 @@ struct NvtxRange {
 #include "mg2d.cuh"
 #include "mgpair2d.cuh"
 #include "mlp.cuh"
+#include "stateio.cuh"
 
 namespace grte2 {
 
@@ -148,6 +149,14 @@ __global__ void k2_acU(D2 D) {
   if (c >= D.g.nc) return;
   const double t = D.T[c];
   D.acU[c] = D.g.a * D.g.c * (t * t) * (t * t);
+}
+
+// E = a c U in every direction (equilibrium)
+__global__ void k2_equilibrium(D2 D) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= D.g.nc) return;
+  const double e = D.g.a * D.g.c * D.U[c];
+  for (int k = 0; k < D.g.K; ++k) D.E[(int64_t)k * D.g.nc + c] = e;
 }
 
 // ----------------------------------------------------------------------------- stencils
@@ -1074,6 +1083,11 @@ static void s8_pairs(std::vector<double>& mu, std::vector<double>& eta, std::vec
 
 // =============================================================================== host
 using namespace grte2;
+using grte::io_block;
+using grte::io_grid;
+using grte::k_fourth_power;
+using grte::k_lines_in;
+using grte::k_lines_out;
 
 // Kernel launches made by this thread (every launch site increments it); grte2d_step
 // reports the difference over the call in grte_stats_t.launches.
@@ -1090,6 +1104,7 @@ struct grte2d_ctx {
   std::vector<void*> allocs;
   std::string err;
   grte_stats_t stats{};
+  double* pin = nullptr;   // pinned: what the host reads back (Hessenberg column, status)
   int host_flags = 0;   // statuses found on the host (a solve that missed its tolerance)
   int m = 30;
   double *V = nullptr, *phi = nullptr, *GU = nullptr, *Es = nullptr;
@@ -1424,8 +1439,9 @@ static grte_status arnoldi_step(grte2d_t h, bool pred, bool mg_stage, S* V, int 
     }
   }
   CK2(cudaGetLastError());
-  CK2(cudaMemcpyAsync(hc.data(), h->hcol, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, st));
+  CK2(cudaMemcpyAsync(h->pin, h->hcol, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, st));
   CK2(cudaStreamSynchronize(st));
+  std::copy(h->pin, h->pin + j + 2, hc.begin());
   return GRTE_OK;
 }
 
@@ -1647,6 +1663,7 @@ void grte2d_destroy(grte2d_t h) {
   if (!h) return;
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->mp_graph) cudaGraphExecDestroy(h->mp_graph);
+  if (h->pin) cudaFreeHost(h->pin);
   for (void* p : h->allocs) cudaFree(p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
@@ -1739,6 +1756,8 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
             alloc2(h, &h->coef, kMaxRestart2 + 1) && alloc2(h, &h->cscale, nc) &&
             alloc2(h, &h->hcol, kMaxRestart2 + 2) && alloc2(h, &h->tk, K * nc);
   if (!ok) return fail2(h, GRTE_ENOMEM, "cudaMalloc failed");
+  if (cudaMallocHost(&h->pin, sizeof(double) * (kMaxRestart2 + 2)) != cudaSuccess)
+    return fail2(h, GRTE_ENOMEM, "cudaMallocHost failed");
   if (h->opt.prec2d & ~(GRTE_PREC2D_MULTIGRID | GRTE_PREC2D_CORR_MG))
     return fail2(h, GRTE_EINVAL, "prec2d: a set of GRTE_PREC2D_MULTIGRID and GRTE_PREC2D_CORR_MG");
   if (h->opt.prec2d & GRTE_PREC2D_CORR_MG) {
@@ -1818,22 +1837,24 @@ grte_status grte2d_set_state(grte2d_t h, const double* T, const double* E, const
   if ((E == nullptr) != (O == nullptr)) return fail2(h, GRTE_EINVAL, "E and O must both be given or both NULL");
   const G2& g = h->g;
   const int64_t K = g.K, nc = g.nc, nv = g.nv;
-  std::vector<double> hE(K * nc), hO(K * nv, 0.0), hU(nc);
-  for (int64_t c = 0; c < nc; ++c) {
+  for (int64_t c = 0; c < nc; ++c)
     if (!(T[c] >= 0.0) || !std::isfinite(T[c])) return fail2(h, GRTE_EINVAL, "T must be finite and >= 0");
-    hU[c] = (T[c] * T[c]) * (T[c] * T[c]);
-  }
-  for (int64_t k = 0; k < K; ++k) {
-    for (int64_t c = 0; c < nc; ++c) hE[k * nc + c] = E ? E[c * K + k] : g.a * g.c * hU[c];
-    if (O)
-      for (int64_t v = 0; v < nv; ++v) hO[k * nv + v] = O[v * K + k];
-  }
   D2& D = h->D;
-  CK2(cudaStreamSynchronize(h->stream));
-  CK2(cudaMemcpy(D.T, T, sizeof(double) * nc, cudaMemcpyHostToDevice));
-  CK2(cudaMemcpy(D.U, hU.data(), sizeof(double) * nc, cudaMemcpyHostToDevice));
-  CK2(cudaMemcpy(D.E, hE.data(), sizeof(double) * K * nc, cudaMemcpyHostToDevice));
-  CK2(cudaMemcpy(D.O, hO.data(), sizeof(double) * K * nv, cudaMemcpyHostToDevice));
+  cudaStream_t st = h->stream;
+  CK2(cudaMemcpyAsync(D.T, T, sizeof(double) * nc, cudaMemcpyHostToDevice, st));
+  k_fourth_power<<<grid_of(nc), kThreads, 0, st>>>(D.T, D.U, nc);
+  if (E) {
+    // the arrays in the host's layout pass through the Krylov basis, free between solves
+    CK2(cudaMemcpyAsync(h->Kbasis, E, sizeof(double) * K * nc, cudaMemcpyHostToDevice, st));
+    k_lines_in<double><<<io_grid(nc, (int)K), io_block(), 0, st>>>(h->Kbasis, D.E, nc, (int)K, nullptr, 0.0);
+    CK2(cudaMemcpyAsync(h->Kbasis, O, sizeof(double) * K * nv, cudaMemcpyHostToDevice, st));
+    k_lines_in<double><<<io_grid(nv, (int)K), io_block(), 0, st>>>(h->Kbasis, D.O, nv, (int)K, nullptr, 0.0);
+  } else {
+    k2_equilibrium<<<grid_of(nc), kThreads, 0, st>>>(D);
+    CK2(cudaMemsetAsync(D.O, 0, sizeof(double) * K * nv, st));
+  }
+  CK2(cudaGetLastError());
+  CK2(cudaStreamSynchronize(st));
   CK2(cudaMemset(D.status, 0, sizeof(int)));
   h->host_flags = 0;
   h->state_set = true;
@@ -1841,9 +1862,9 @@ grte_status grte2d_set_state(grte2d_t h, const double* T, const double* E, const
 }
 
 static grte_status status2(grte2d_t h) {
-  int s = 0;
+  CK2(cudaMemcpyAsync(h->pin, h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CK2(cudaStreamSynchronize(h->stream));
-  CK2(cudaMemcpy(&s, h->D.status, sizeof(int), cudaMemcpyDeviceToHost));
+  int s = *(const int*)h->pin;
   s |= h->host_flags;
   h->stats.status_flags = s;
   for (int code : {GRTE_ENAN, GRTE_ENONCONV, GRTE_ENEGATIVE, GRTE_ETIMEOUT})
@@ -1871,9 +1892,16 @@ grte_status grte2d_step(grte2d_t h, int64_t n) {
 
 static grte_status get2(grte2d_t h, const double* src, int64_t count, double* out, size_t len) {
   if (!out || len != (size_t)count) return fail2(h, GRTE_EINVAL, "bad output length");
-  CK2(cudaStreamSynchronize(h->stream));
-  CK2(cudaMemcpy(out, src, sizeof(double) * count, cudaMemcpyDeviceToHost));
+  CK2(cudaMemcpyAsync(out, src, sizeof(double) * count, cudaMemcpyDeviceToHost, h->stream));
   return status2(h);
+}
+
+// K lines of `rows` values in the host's layout, through the Krylov basis (free between solves)
+static grte_status get_lines2(grte2d_t h, const double* src, int64_t rows, double* out) {
+  const int K = h->g.K;
+  k_lines_out<double><<<io_grid(rows, K), io_block(), 0, h->stream>>>(src, h->Kbasis, rows, K, nullptr, 0.0);
+  CK2(cudaGetLastError());
+  return get2(h, h->Kbasis, rows * K, out, (size_t)(rows * K));
 }
 
 grte_status grte2d_get_T(grte2d_t h, double* T, size_t len) {
@@ -1885,22 +1913,14 @@ grte_status grte2d_get_E(grte2d_t h, double* E, size_t len) {
   if (!h) return GRTE_EINVAL;
   const int64_t K = h->g.K, nc = h->g.nc;
   if (!E || len != (size_t)(K * nc)) return fail2(h, GRTE_EINVAL, "len must be nx*ny*K");
-  std::vector<double> t(K * nc);
-  grte_status s = get2(h, h->D.E, K * nc, t.data(), t.size());
-  for (int64_t k = 0; k < K; ++k)
-    for (int64_t c = 0; c < nc; ++c) E[c * K + k] = t[k * nc + c];
-  return s;
+  return get_lines2(h, h->D.E, nc, E);
 }
 
 grte_status grte2d_get_O(grte2d_t h, double* O, size_t len) {
   if (!h) return GRTE_EINVAL;
   const int64_t K = h->g.K, nv = h->g.nv;
   if (!O || len != (size_t)(K * nv)) return fail2(h, GRTE_EINVAL, "len must be (nx+1)*(ny+1)*K");
-  std::vector<double> t(K * nv);
-  grte_status s = get2(h, h->D.O, K * nv, t.data(), t.size());
-  for (int64_t k = 0; k < K; ++k)
-    for (int64_t v = 0; v < nv; ++v) O[v * K + k] = t[k * nv + v];
-  return s;
+  return get_lines2(h, h->D.O, nv, O);
 }
 
 grte_status grte2d_get_stage(grte2d_t h, int which, double* out, size_t len) {

