@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/grte.h"
@@ -47,7 +48,6 @@ constexpr int kMaxPairs = 64;
 constexpr int kMaxRestart2 = 64;
 constexpr int kThreads = 256;
 constexpr int kRedBlocks = 304;   // 2 x 152 SMs: blocks of the first reduction stage
-constexpr int kDotBlocks = 304;   // 2 x 152: blocks of the Gram-Schmidt dot products (one wave)
 constexpr int kAxpyBlocks = 1216; // 8 x 152: blocks of the streaming vector updates
 
 struct G2 {
@@ -136,19 +136,33 @@ __global__ void k2_vcoef(D2 D) {
   D.odv[v] = d * g.eps * g.eps / (g.c * g.dt);
 }
 
+// T^4 to half an ulp (the square's rounding error carried along): an equilibrium state then
+// meets the walls' intensity a c T^4 exactly, which the wall rows multiply by 2/eps.
+__device__ __forceinline__ double fourth_power(double t) {
+  const double p = t * t, e = fma(t, t, -p);
+  return fma(p, p, 2.0 * p * e);
+}
+
+__global__ void k2_fourth_power(D2 D) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c < D.g.nc) D.U[c] = fourth_power(D.T[c]);
+}
+
+// rho = sum_k w_k E_k as E_0 + sum_k w_k (E_k - E_0) (sum_k w_k = 1): exact in equilibrium,
+// where the plain sum is an ulp or two off and the wall rows multiply that by 2/eps.
 __global__ void k2_rho(D2 D, const double* __restrict__ E, double* __restrict__ out) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= D.g.nc) return;
+  const double e0 = E[c];
   double r = 0.0;
-  for (int k = 0; k < D.g.K; ++k) r += D.w[k] * E[(int64_t)k * D.g.nc + c];
-  out[c] = r;
+  for (int k = 1; k < D.g.K; ++k) r += D.w[k] * (E[(int64_t)k * D.g.nc + c] - e0);
+  out[c] = e0 + r;
 }
 
 __global__ void k2_acU(D2 D) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= D.g.nc) return;
-  const double t = D.T[c];
-  D.acU[c] = D.g.a * D.g.c * (t * t) * (t * t);
+  D.acU[c] = D.g.a * D.g.c * fourth_power(D.T[c]);
 }
 
 // E = a c U in every direction (equilibrium)
@@ -173,18 +187,17 @@ struct CV {
   S h2x, h2y, te;
 };
 
-// Per-pair cell field u_k(c) = (uk[k*ks + c] + ub[c]) * sc[c] (any part may be absent).
+// Per-pair cell field u_k(c) = uk[k*ks + c] + ub[c] (either part may be absent).
 template <typename S>
 struct UFieldT {
   const S* uk;
   int64_t ks;
   const S* ub;
-  const S* sc = nullptr;
   __device__ __forceinline__ S at(int k, int c) const {
     S v = S(0);
     if (uk) v += uk[(int64_t)k * ks + c];
     if (ub) v += ub[c];
-    return sc ? v * sc[c] : v;
+    return v;
   }
   __device__ __forceinline__ bool any() const { return uk || ub; }
 };
@@ -288,7 +301,7 @@ __global__ void k2_wallshift(D2 D, double* __restrict__ V, const double* __restr
   V[t] = Vp[t] + (V[vin] - Vp[vin]);
 }
 
-enum { C_MV_PRED = 0, C_MV_CORR = 1, C_DIVK = 2, C_FDIV = 3 };
+enum { C_DIVK = 0, C_FDIV = 1 };
 
 // Side weights of cell (p, q) for pair k: the streaming derivative of O at the cell is
 //   mu/(2 dx) [wL (O00 + O01) + wR (O10 + O11)] + eta/(2 dy) [wB (O00 + O10) + wT (O01 + O11)]
@@ -296,31 +309,32 @@ enum { C_MV_PRED = 0, C_MV_CORR = 1, C_DIVK = 2, C_FDIV = 3 };
 // with (wL, wR, wB, wT) = (-1, 1, -1, 1) inside.  A cell beside an inflow wall applies
 // Eq. bc-pre to its own wall side as the 1D wall cell does: the low x side becomes
 // s 2/eps (b - E_cell) - (high side), i.e. mu (2 R - s 2/eps (b - E_cell))/dx, and
-// likewise for the other sides (s = +1 if Omega_k enters there, else -1).
+// likewise for the other sides (s = +1 if Omega_k enters there, else -1).  The wall sides' own
+// terms are ex (E_cell - bx) + ey (E_cell - by); ed = ex + ey multiplies E_cell alone.
 template <typename S>
 struct CellSides {
-  S wL, wR, wB, wT, ed, bt;
+  S wL, wR, wB, wT, ex, ey, bx, by;
+  __device__ __forceinline__ S ed() const { return ex + ey; }
 };
 
 template <typename S>
 __device__ __forceinline__ CellSides<S> cell_sides(const D2& D, const CV<S>& cv, int k, int p, int q) {
   const G2& g = D.g;
-  CellSides<S> cs{S(-1), S(1), S(-1), S(1), S(0), S(0)};
+  CellSides<S> cs{S(-1), S(1), S(-1), S(1), S(0), S(0), S(0), S(0)};
   const S mu = cv.mu[k], eta = cv.eta[k], te = cv.te, ix = S(2) * cv.h2x, iy = S(2) * cv.h2y;
-  if (g.bcx == GRTE_BC_INFLOW) {
+  if (g.bcx == GRTE_BC_INFLOW) {   // (Nx, Ny >= 2: a cell has at most one wall per axis)
     if (p == 0) {
       const S s = mu > S(0) ? S(1) : S(-1);   // Omega_k enters at x = 0 when mu > 0
       cs.wL = S(0);
       cs.wR = S(2);
-      cs.ed += mu * s * te * ix;
-      cs.bt -= mu * s * te * S(g.bx0) * ix;
-    }
-    if (p == g.Nx - 1) {
+      cs.ex = mu * s * te * ix;
+      cs.bx = S(g.bx0);
+    } else if (p == g.Nx - 1) {
       const S s = mu < S(0) ? S(1) : S(-1);
-      if (p != 0) cs.wL = S(-2);
+      cs.wL = S(-2);
       cs.wR = S(0);
-      cs.ed -= mu * s * te * ix;
-      cs.bt += mu * s * te * S(g.bx1) * ix;
+      cs.ex = -(mu * s * te * ix);
+      cs.bx = S(g.bx1);
     }
   }
   if (g.bcy == GRTE_BC_INFLOW) {
@@ -328,15 +342,14 @@ __device__ __forceinline__ CellSides<S> cell_sides(const D2& D, const CV<S>& cv,
       const S s = eta > S(0) ? S(1) : S(-1);
       cs.wB = S(0);
       cs.wT = S(2);
-      cs.ed += eta * s * te * iy;
-      cs.bt -= eta * s * te * S(g.by0) * iy;
-    }
-    if (q == g.Ny - 1) {
+      cs.ey = eta * s * te * iy;
+      cs.by = S(g.by0);
+    } else if (q == g.Ny - 1) {
       const S s = eta < S(0) ? S(1) : S(-1);
-      if (q != 0) cs.wB = S(-2);
+      cs.wB = S(-2);
       cs.wT = S(0);
-      cs.ed -= eta * s * te * iy;
-      cs.bt += eta * s * te * S(g.by1) * iy;
+      cs.ey = -(eta * s * te * iy);
+      cs.by = S(g.by1);
     }
   }
   return cs;
@@ -359,8 +372,10 @@ __device__ __forceinline__ S cell_div(const D2& D, const CV<S>& cv, const S* __r
   const CellSides<S> cs = cell_sides<S>(D, cv, k, p, q);
   S div = cv.mu[k] * cv.h2x * (cs.wL * (Vk[v00] + Vk[v01]) + cs.wR * (Vk[v10] + Vk[v11])) +
           cv.eta[k] * cv.h2y * (cs.wB * (Vk[v00] + Vk[v10]) + cs.wT * (Vk[v01] + Vk[v11]));
-  if (u.any()) div += cs.ed * u.at(k, (int)c);
-  if constexpr (DATA) div += cs.bt;
+  // with field and data the difference E - b is taken first: 2/eps multiplies it
+  const S e = u.any() ? u.at(k, (int)c) : S(0);
+  if constexpr (DATA) div += cs.ex * (e - cs.bx) + cs.ey * (e - cs.by);
+  else div += cs.ed() * e;
   return div;
 }
 
@@ -388,21 +403,14 @@ __global__ void k2_fdiv_corr(D2 D, CV<double> cv, const double* __restrict__ V, 
   const CellSides<double> cs = cell_sides<double>(D, cv, k, p, q);
   tk[t] = cv.mu[k] * cv.h2x * (cs.wL * (Vx[v00] + Vx[v01]) + cs.wR * (Vx[v10] + Vx[v11])) +
           cv.eta[k] * cv.h2y * (cs.wB * (Vy[v00] + Vy[v10]) + cs.wT * (Vy[v01] + Vy[v11])) +
-          cs.ed * u.at(k, ci) + cs.bt;
+          cs.ex * (u.at(k, ci) - cs.bx) + cs.ey * (u.at(k, ci) - cs.by);
 }
 
 // Cell pass over the vertex values V (computed from the same field u, with the data
-// part when DATA), one thread per (pair, cell):
-//   C_MV_PRED: y_k = A z_k + alpha z_rho + kappa S_k,  t_k = kappa S_k (for the rho row)
-//   C_MV_CORR: y_k = A z_k + kappa S_k
-//   C_DIVK:    y_k = kappa S_k
-//   C_FDIV:    t_k = S_k
-// S_k the streaming derivative of O_k at the cell (cell_sides).  z is read scaled by
-// zs[c] when zs is given (the Krylov unknowns are cell-scaled).  The sums over pairs
-// (rho row, C_FDIV) are k2_cellsum.
+// part when DATA), one thread per (pair, cell): C_DIVK: y_k = kappa S_k, C_FDIV: y_k = S_k,
+// S_k the streaming derivative of O_k at the cell (cell_sides).
 template <typename S, int MODE, bool DATA>
-__global__ void k2_cell(D2 D, CV<S> cv, const S* __restrict__ V, UFieldT<S> u, const S* __restrict__ z,
-                        S* __restrict__ y, const S* __restrict__ zs, S* __restrict__ tk) {
+__global__ void k2_cell(D2 D, CV<S> cv, const S* __restrict__ V, UFieldT<S> u, S* __restrict__ y) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const G2& g = D.g;
   if (t >= (int64_t)g.K * g.nc) return;
@@ -410,36 +418,17 @@ __global__ void k2_cell(D2 D, CV<S> cv, const S* __restrict__ V, UFieldT<S> u, c
   const int k = tt / nc;
   const int64_t c = tt - k * nc;
   const S div = cell_div<S, DATA>(D, cv, V, u, k, c);
-  const S kc = cv.kc[c];
-  const S f = zs ? zs[c] : S(1);
-  if (MODE == C_MV_PRED) {
-    y[t] = cv.A[c] * f * z[t] + cv.alpha[c] * f * z[(int64_t)g.K * g.nc + c] + kc * div;
-    tk[t] = kc * div;
-  } else if (MODE == C_MV_CORR) {
-    y[t] = cv.A[c] * f * z[t] + kc * div;
-  } else if (MODE == C_DIVK) {
-    y[t] = kc * div;
-  } else {
-    tk[t] = div;
-  }
+  y[t] = MODE == C_DIVK ? cv.kc[c] * div : div;
 }
 
-// Per-cell sums over pairs (fixed order): C_MV_PRED: y_rho = alpha z_rho + sum_k w_k t_k;
-// C_FDIV: y = sum_k w_k t_k.
-template <typename S, int MODE>
-__global__ void k2_cellsum(D2 D, CV<S> cv, const S* __restrict__ tk, const S* __restrict__ z, S* __restrict__ y,
-                           const S* __restrict__ zs) {
+// sum_k w_k t_k per cell (fixed order)
+__global__ void k2_cellsum(D2 D, const double* __restrict__ tk, double* __restrict__ y) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const G2& g = D.g;
   if (c >= g.nc) return;
-  S acc = S(0);
-  for (int k = 0; k < g.K; ++k) acc += cv.w[k] * tk[(int64_t)k * g.nc + c];
-  if (MODE == C_MV_PRED) {
-    const S f = zs ? zs[c] : S(1);
-    y[(int64_t)g.K * g.nc + c] = cv.alpha[c] * f * z[(int64_t)g.K * g.nc + c] + acc;
-  } else {
-    y[c] = acc;
-  }
+  double acc = 0.0;
+  for (int k = 0; k < g.K; ++k) acc += D.w[k] * tk[(int64_t)k * g.nc + c];
+  y[c] = acc;
 }
 
 // Diagonal of G_k at cell c (for the preconditioner): the node-equation vertices of
@@ -456,7 +445,7 @@ __device__ double gdiag(const D2& D, const CV<double>& cv, int k, int p, int q) 
                          cs.wR * mx + cs.wT * ey};
   const double a = mx + ey, b = mx - ey;
   const double cgr[4] = {a, -b, b, -a};   // D_k coefficient of this cell at vertex t
-  double r = cs.ed;
+  double r = cs.ed();
   for (int t = 0; t < 4; ++t) {
     const int i = p + di[t], j = q + dj[t];
     if (vkind(g, i, j) != 0) continue;
@@ -464,37 +453,6 @@ __device__ double gdiag(const D2& D, const CV<double>& cv, int k, int p, int q) 
     r += cst[t] * (-D.dv[v] * cgr[t]);
   }
   return D.kc[q * g.Nx + p] * r;
-}
-
-// Left preconditioner.  Prediction: per cell, the angular block of the matrix with G_k
-// replaced by its diagonal g_k (an arrow matrix), solved exactly:
-//   rho = [r_rho - sum_k w_k g_k r_k/(A+g_k)] / [alpha + sum_k w_k g_k (A - alpha)/(A+g_k)],
-//   e_k = (r_k - (alpha + g_k) rho)/(A + g_k).
-// Correction: z_k = r_k/(A + g_k).  The result is multiplied by the cell's Krylov
-// scale w (the GMRES runs on w-scaled unknowns: D_w P^{-1} M D_w^{-1}).
-// (the diagonals g_k and the reciprocals come from k2_gdiag, once per solve)
-template <typename S, bool PRED>
-__global__ void k2_prec(D2 D, CV<S> cv, const S* __restrict__ r, S* __restrict__ z) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const G2& g = D.g;
-  if (c >= g.nc) return;
-  const S ws = cv.wsc[c];
-  if (!PRED) {
-    for (int k = 0; k < g.K; ++k) z[(int64_t)k * g.nc + c] = ws * r[(int64_t)k * g.nc + c] * cv.gdi[(int64_t)k * g.nc + c];
-    return;
-  }
-  const S al = cv.alpha[c];
-  S num = r[(int64_t)g.K * g.nc + c];
-  for (int k = 0; k < g.K; ++k) {
-    const int64_t o = (int64_t)k * g.nc + c;
-    num -= cv.w[k] * cv.gd[o] * r[o] * cv.gdi[o];
-  }
-  const S rho = num * cv.pdi[c];
-  z[(int64_t)g.K * g.nc + c] = ws * rho;
-  for (int k = 0; k < g.K; ++k) {
-    const int64_t o = (int64_t)k * g.nc + c;
-    z[o] = ws * (r[o] - (al + cv.gd[o]) * rho) * cv.gdi[o];
-  }
 }
 
 // ----------------------------------------------------------------------------- Schur preconditioner
@@ -659,48 +617,11 @@ __global__ void k2_gdiag(D2 D, CV<double> cv) {
   D.pdi[c] = 1.0 / den;
 }
 
-// Krylov scale per cell from a magnitude field src: s = |src| + 1e-13 max|src| (or
-// s = max|src| for every cell with uniform), w = f/s (f = 1 in the prediction, eps in the correction, whose unknown E_J enters
-// E as eps E_J).
-__global__ void k2_maxabs(const double* __restrict__ x, int64_t n, double* __restrict__ part) {
-  __shared__ double red[kThreads / 32];
-  double t = 0.0;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    t = fmax(t, fabs(x[j]));
-  for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) m = fmax(m, red[q]);
-    part[blockIdx.x] = m;
-  }
-}
-
-__global__ void k2_weights(D2 D, const double* __restrict__ src, double f, const double* __restrict__ part, int nb,
-                           int uniform) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= D.g.nc) return;
-  double m = 0.0;
-  for (int b = 0; b < nb; ++b) m = fmax(m, part[b]);
-  const double s = (uniform ? m : fabs(src[c]) + 1e-13 * m) + 1e-300;
-  D.wsc[c] = f / s;
-  D.iwsc[c] = s / f;
-}
-
 // magnitude of E^{n+1} per cell for the correction's scale: max(a c U, |rho*|)
 __global__ void k2_corrscale(D2 D, double* __restrict__ out) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= D.g.nc) return;
   out[c] = fmax(D.acU[c], fabs(D.rho_s[c]));
-}
-
-// x[k][c] *= sc[c] over nvec stacked per-cell blocks
-__global__ void k2_cellscale(double* __restrict__ x, const double* __restrict__ sc, int nvec, int64_t nc) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= nc) return;
-  const double f = sc[c];
-  for (int k = 0; k < nvec; ++k) x[(int64_t)k * nc + c] *= f;
 }
 
 // ----------------------------------------------------------------------------- right-hand sides
@@ -767,8 +688,7 @@ __global__ void k2_project(D2 D, const double* __restrict__ EJ) {
     const int64_t o = (int64_t)k * g.nc + c;
     D.E[o] = acU + g.eps * EJ[o];
   }
-  const double t = D.T[c];
-  D.U[c] = (t * t) * (t * t);
+  D.U[c] = fourth_power(D.T[c]);
 }
 
 // ----------------------------------------------------------------------------- Newton
@@ -847,47 +767,7 @@ __global__ void k2_newton(D2 D) {
 }
 
 // ----------------------------------------------------------------------------- vector kernels
-// Partial dot products of w with V_0..V_{nvec-1} (stride n): one value per (block, vec),
-// fixed order; k2_reduce sums the block partials (one block per value).  The vectors go
-// in chunks of C (w read once per chunk), each thread keeping C sums in the vectors'
-// precision S; the block sums are binary64.  All C loads of an element are issued
-// unconditionally (a chunk's missing vectors read its last one and are masked out), so
-// they are in flight together; the warp sums are formed in S and widened once.
-template <typename S, int C>
-__global__ void __launch_bounds__(kThreads, 2) k2_mdot(const S* __restrict__ w, const S* __restrict__ V, int nvec,
-                                                     int64_t n, double* __restrict__ part) {
-  __shared__ double red[kThreads / 32][C];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int i0 = 0; i0 < nvec; i0 += C) {
-    const int nv = min(C, nvec - i0);
-    const S* Vb = V + (int64_t)i0 * n;
-    S acc[C];
-#pragma unroll
-    for (int t = 0; t < C; ++t) acc[t] = S(0);
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-      const S wj = w[j];
-      S vt[C];
-#pragma unroll
-      for (int t = 0; t < C; ++t) vt[t] = Vb[(int64_t)min(t, nv - 1) * n + j];
-#pragma unroll
-      for (int t = 0; t < C; ++t) acc[t] = t < nv ? fma(wj, vt[t], acc[t]) : acc[t];
-    }
-#pragma unroll
-    for (int t = 0; t < C; ++t) {
-      S v = acc[t];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[wid][t] = (double)v;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nv; t += blockDim.x) {
-      double u = 0.0;
-      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) u += red[q][t];
-      part[(int64_t)(i0 + t) * gridDim.x + blockIdx.x] = u;
-    }
-    __syncthreads();
-  }
-}
-
+// one block per value: the sum of its nb block parts
 __global__ void k2_reduce(const double* __restrict__ part, int nb, double* __restrict__ out) {
   __shared__ double red[kThreads / 32];
   double t = 0.0;
@@ -902,98 +782,10 @@ __global__ void k2_reduce(const double* __restrict__ part, int nb, double* __res
   }
 }
 
-// k2_reduce for the Gram-Schmidt coefficients: coef[b] = sum of value b's partials and
-// the Hessenberg column hcol[b] (+)= coef[b] (first pass: assign)
-__global__ void k2_reduce_h(const double* __restrict__ part, int nb, double* __restrict__ coef,
-                            double* __restrict__ hcol, int assign) {
-  __shared__ double red[kThreads / 32];
-  double t = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) t += part[(int64_t)blockIdx.x * nb + b];
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += red[q];
-    coef[blockIdx.x] = s;
-    hcol[blockIdx.x] = assign ? s : hcol[blockIdx.x] + s;
-  }
-}
-
-// w -= sum_i coef[i] V_i (coefficients staged in shared memory in the vectors' precision,
-// four independent partial sums per element); with NORM also the block partials of
-// |w|^2 of the result (binary64).
-template <typename S, bool NORM>
-__global__ void __launch_bounds__(kThreads) k2_maxpy(S* __restrict__ w, const S* __restrict__ V,
-                                                      const double* __restrict__ coef, int nvec, int64_t n,
-                                                      double* __restrict__ part) {
-  __shared__ S cf[kMaxRestart2 + 1];
-  __shared__ double red[kThreads / 32];
-  for (int i = threadIdx.x; i < nvec; i += blockDim.x) cf[i] = S(coef[i]);
-  __syncthreads();
-  S nrm = S(0);
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    S t0 = w[j], t1 = S(0), t2 = S(0), t3 = S(0);
-    int i = 0;
-    for (; i + 4 <= nvec; i += 4) {
-      t0 = fma(-cf[i], V[(int64_t)i * n + j], t0);
-      t1 = fma(-cf[i + 1], V[(int64_t)(i + 1) * n + j], t1);
-      t2 = fma(-cf[i + 2], V[(int64_t)(i + 2) * n + j], t2);
-      t3 = fma(-cf[i + 3], V[(int64_t)(i + 3) * n + j], t3);
-    }
-    for (; i < nvec; ++i) t0 = fma(-cf[i], V[(int64_t)i * n + j], t0);
-    const S r = (t0 + t1) + (t2 + t3);
-    w[j] = r;
-    if (NORM) nrm = fma(r, r, nrm);
-  }
-  if (NORM) {
-    double v = nrm;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double u = 0.0;
-      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) u += red[q];
-      part[blockIdx.x] = u;
-    }
-  }
-}
-
-// x += sum_i coef[i] V_i (x binary64; binary32 basis vectors: the combination is formed
-// in binary32 and added once)
-template <typename S>
-__global__ void k2_update(double* __restrict__ x, const S* __restrict__ V, const double* __restrict__ coef, int nvec,
-                          int64_t n) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    if constexpr (sizeof(S) == 8) {
-      double t = x[j];
-      for (int i = 0; i < nvec; ++i) t += coef[i] * V[(int64_t)i * n + j];
-      x[j] = t;
-    } else {
-      S t = S(0);
-      for (int i = 0; i < nvec; ++i) t = fma(S(coef[i]), V[(int64_t)i * n + j], t);
-      x[j] += (double)t;
-    }
-  }
-}
-
-template <typename S>
-__global__ void k2_scale(S* __restrict__ x, double s, int64_t n) {
-  const S f = S(s);
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    x[j] *= f;
-}
-
 // binary32 copy dst = src * f
 __global__ void k2_tof(const double* __restrict__ src, float* __restrict__ dst, int64_t n, double f) {
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
     dst[j] = (float)(src[j] * f);
-}
-
-// y = b - y
-__global__ void k2_bminus(const double* __restrict__ b, double* __restrict__ y, int64_t n) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    y[j] = b[j] - y[j];
 }
 
 __global__ void k2_energy(D2 D, double* __restrict__ part) {
@@ -1014,6 +806,8 @@ __global__ void k2_energy(D2 D, double* __restrict__ part) {
     part[blockIdx.x] = s;
   }
 }
+
+#include "krylov2d.cuh"
 
 // Level-symmetric S8 pairs for 2D (80 directions on the sphere: cosine levels
 // mu_i^2 = (1 + 6 i)/21, i = 0..3; per octant the permutations of the level triples
@@ -1085,13 +879,15 @@ static void s8_pairs(std::vector<double>& mu, std::vector<double>& eta, std::vec
 using namespace grte2;
 using grte::io_block;
 using grte::io_grid;
-using grte::k_fourth_power;
 using grte::k_lines_in;
 using grte::k_lines_out;
 
 // Kernel launches made by this thread (every launch site increments it); grte2d_step
 // reports the difference over the call in grte_stats_t.launches.
 static thread_local int64_t tl_launches = 0;
+constexpr int kLook = 2;   // Arnoldi steps launched ahead of the last decision seen (gmres2)
+// stride of the basis vectors: 16-byte boundaries for both types
+static int64_t basis_ld(int64_t n) { return (n + 3) / 4 * 4; }
 
 struct grte2d_ctx {
   D2 D{};
@@ -1104,12 +900,15 @@ struct grte2d_ctx {
   std::vector<void*> allocs;
   std::string err;
   grte_stats_t stats{};
-  double* pin = nullptr;   // pinned: what the host reads back (Hessenberg column, status)
+  KPin* pin = nullptr;     // pinned: what the host reads back
+  KState* ks = nullptr;    // the Krylov cycle's scalars (device)
+  unsigned* count = nullptr;   // blocks of a reduction that have arrived
+  cudaEvent_t ev[kLook + 1] = {};   // one per Arnoldi step in flight
   int host_flags = 0;   // statuses found on the host (a solve that missed its tolerance)
   int m = 30;
   double *V = nullptr, *phi = nullptr, *GU = nullptr, *Es = nullptr;
   double *b = nullptr, *x = nullptr, *Kr = nullptr, *Kt = nullptr, *Kbasis = nullptr;
-  double *part = nullptr, *dots = nullptr, *coef = nullptr, *cscale = nullptr, *hcol = nullptr;
+  double *part = nullptr, *dots = nullptr, *cscale = nullptr;
   double* tk = nullptr;   // [k][cell] per-pair cell values summed by k2_cellsum
   grte_mlp_t mlp = nullptr;   // learned Newton start (not owned)
   CV<double> cv{};            // the binary64 coefficient view of D
@@ -1119,7 +918,7 @@ struct grte2d_ctx {
   CV<float> cv32{};
   float *mu32 = nullptr, *eta32 = nullptr, *w32 = nullptr, *kc32 = nullptr, *A32 = nullptr, *alpha32 = nullptr;
   float *dv32 = nullptr, *gd32 = nullptr, *gdi32 = nullptr, *pdi32 = nullptr, *wsc32 = nullptr, *iwsc32 = nullptr;
-  float *V32 = nullptr, *Kr32 = nullptr, *Vv32 = nullptr, *tk32 = nullptr;
+  float *V32 = nullptr, *Kr32 = nullptr;
   std::vector<mg::Level> mgl;        // multigrid levels of the Schur preconditioner (empty: per-cell block only)
   double *mg_M = nullptr, *mg_inv = nullptr;   // coarsest level: dense scratch and inverse
   // correction substep 2: per-pair multigrid (GRTE_PREC2D_CORR_MG), its V-cycle as one graph
@@ -1152,55 +951,82 @@ static bool alloc2(grte2d_t h, T** p, int64_t n) {
   return true;
 }
 
+// The operator pass (k2_op).  Tiles of 32 x 8 cells with one thread per cell and all pairs in
+// turn have the least halo and are the cheapest per cell; where they are too few to fill the
+// chip, tiles of 32 x 4 whose pairs are shared by four groups of threads; and 8 x 4 with ten
+// groups where those are few, too: a small grid waits for the pairs' chain of barriers and
+// wants its binary64 work spread over all SMs.
+template <typename S, bool PRED, bool PREC, bool RES, int TX, int TY, int G>
+static void op_launch(grte2d_t h, const CV<S>& cv, const S* z, const S* sc, const double* inv, const S* b, S* out,
+                      const int* stop) {
+  const G2& g = h->D.g;
+  const dim3 grid((unsigned)((g.Nx + TX - 1) / TX), (unsigned)((g.Ny + TY - 1) / TY));
+  k2_op<S, PRED, PREC, RES, TX, TY, G><<<grid, TX * TY * G, op_smem<S>(g.K, TX, TY, G, PREC && PRED), h->stream>>>(
+      h->D, cv, z, sc, inv, b, out, stop);
+  tl_launches++;
+}
+static int64_t op_tiles(const G2& g, int tx, int ty) {
+  return (int64_t)((g.Nx + tx - 1) / tx) * ((g.Ny + ty - 1) / ty);
+}
+template <typename S, bool PREC, bool RES>
+static void op_pass(grte2d_t h, bool pred, const CV<S>& cv, const S* z, const S* sc, const double* inv, const S* b,
+                    S* out, const int* stop) {
+  const G2& g = h->D.g;
+  auto go = [&](auto P) {
+    constexpr bool PR = decltype(P)::value;
+    if (op_tiles(g, 32, 8) >= 4 * 152) op_launch<S, PR, PREC, RES, 32, 8, 1>(h, cv, z, sc, inv, b, out, stop);
+    else if (op_tiles(g, 32, 4) >= 152) op_launch<S, PR, PREC, RES, 32, 4, 4>(h, cv, z, sc, inv, b, out, stop);
+    else op_launch<S, PR, PREC, RES, 8, 4, 10>(h, cv, z, sc, inv, b, out, stop);
+  };
+  if (pred) go(std::true_type{});
+  else go(std::false_type{});
+}
+
+// The vector kernels' blocks for n values: four 16-byte groups per thread, at most four blocks
+// per SM.
+static unsigned vec_blocks(int64_t n, size_t es) {
+  const int64_t groups = n / (int64_t)(16 / es) + 1;
+  return (unsigned)std::min<int64_t>((groups + 4 * kThreads - 1) / (4 * kThreads), kVecBlocks);
+}
 template <typename S>
-static void launch_mdot(const S* w, const S* V, int nvec, int64_t n, double* part, cudaStream_t st) {
-  if (nvec <= 4) tl_launches++, k2_mdot<S, 4><<<kDotBlocks, kThreads, 0, st>>>(w, V, nvec, n, part);
-  else if (nvec <= 8) tl_launches++, k2_mdot<S, 8><<<kDotBlocks, kThreads, 0, st>>>(w, V, nvec, n, part);
-  else tl_launches++, k2_mdot<S, 16><<<kDotBlocks, kThreads, 0, st>>>(w, V, nvec, n, part);
+static void dot_launch(grte2d_t h, const S* w, const S* V, int64_t ld, int nv, int64_t n, int pass) {
+  const unsigned nb = vec_blocks(n, sizeof(S));
+  auto go = [&](auto C, int per_sm) {
+    k2_dot<S, decltype(C)::value><<<std::min<unsigned>(nb, per_sm * 152), kThreads, 0, h->stream>>>(
+        w, V, ld, nv, n, h->part, h->ks, h->count, pass, h->pin);
+    tl_launches++;
+  };
+  if (nv <= 3) go(std::integral_constant<int, 4>{}, 4);
+  else if (nv <= 7) go(std::integral_constant<int, 8>{}, 3);
+  else go(std::integral_constant<int, 16>{}, 2);
 }
 
-// dots[i] = <w, V_i>, i < nvec, returned on the host.
-static grte_status mdot(grte2d_t h, const double* w, const double* V, int nvec, int64_t n, double* host) {
-  cudaStream_t st = h->stream;
-  launch_mdot<double>(w, V, nvec, n, h->part, st);
-  tl_launches++, k2_reduce<<<nvec, kThreads, 0, st>>>(h->part, kDotBlocks, h->dots);
-  CK2(cudaGetLastError());
-  CK2(cudaMemcpyAsync(host, h->dots, sizeof(double) * nvec, cudaMemcpyDeviceToHost, st));
-  CK2(cudaStreamSynchronize(st));
-  return GRTE_OK;
+template <typename S, bool PRED, bool PREC, bool RES>
+static cudaError_t op_attr(int bytes) {
+  const auto set = [&](const void* f) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+  cudaError_t e = set((const void*)k2_op<S, PRED, PREC, RES, 32, 8, 1>);
+  if (e == cudaSuccess) e = set((const void*)k2_op<S, PRED, PREC, RES, 32, 4, 4>);
+  if (e == cudaSuccess) e = set((const void*)k2_op<S, PRED, PREC, RES, 8, 4, 10>);
+  return e;
 }
-
-// y = M x (pred: the (e, rho) matrix; corr: the stacked A + G_k), through the vertex
-// and cell passes.  The Krylov unknowns are w-scaled: they are unscaled on the way in.
-static void apply_M(grte2d_t h, bool pred, const double* xin, double* y) {
-  D2& D = h->D;
-  cudaStream_t st = h->stream;
-  UField u{xin, D.g.nc, pred ? xin + (int64_t)D.g.K * D.g.nc : nullptr, D.iwsc};
-  const int64_t K = D.g.K;
-  tl_launches++, k2_vertex<double, false><<<grid_of(K * D.g.nv), kThreads, 0, st>>>(D, h->cv, u, h->V);
-  if (pred) {
-    tl_launches++, k2_cell<double, C_MV_PRED, false><<<grid_of(K * D.g.nc), kThreads, 0, st>>>(D, h->cv, h->V, u, xin, y, D.iwsc, h->tk);
-    tl_launches++, k2_cellsum<double, C_MV_PRED><<<grid_of(D.g.nc), kThreads, 0, st>>>(D, h->cv, h->tk, xin, y, D.iwsc);
-  } else {
-    tl_launches++, k2_cell<double, C_MV_CORR, false><<<grid_of(K * D.g.nc), kThreads, 0, st>>>(D, h->cv, h->V, u, xin, y, D.iwsc, h->tk);
-  }
-}
-
-// binary32 matrix and block preconditioner (mixed precision Krylov cycles)
-static void apply_M32(grte2d_t h, bool pred, const float* xin, float* y) {
-  D2& D = h->D;
-  cudaStream_t st = h->stream;
-  const int64_t K = D.g.K, nc = D.g.nc;
-  UFieldT<float> u{xin, nc, pred ? xin + K * nc : nullptr, h->cv32.iwsc};
-  tl_launches++, k2_vertex<float, false><<<grid_of(K * D.g.nv), kThreads, 0, st>>>(D, h->cv32, u, h->Vv32);
-  if (pred) {
-    tl_launches++, k2_cell<float, C_MV_PRED, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv32, h->Vv32, u, xin, y,
-                                                                         h->cv32.iwsc, h->tk32);
-    tl_launches++, k2_cellsum<float, C_MV_PRED><<<grid_of(nc), kThreads, 0, st>>>(D, h->cv32, h->tk32, xin, y, h->cv32.iwsc);
-  } else {
-    tl_launches++, k2_cell<float, C_MV_CORR, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv32, h->Vv32, u, xin, y,
-                                                                         h->cv32.iwsc, h->tk32);
-  }
+// The operator kernels' shared-memory limit (kMaxPairs binary64 pairs need 166 KB).
+static cudaError_t op_attrs() {
+  int dev = 0, bytes = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = op_attr<double, true, true, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, false, true, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, true, true, true>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, false, true, true>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, true, false, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, false, false, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, true, false, true>(bytes);
+  if (e == cudaSuccess) e = op_attr<double, false, false, true>(bytes);
+  if (e == cudaSuccess) e = op_attr<float, true, true, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<float, false, true, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<float, true, false, false>(bytes);
+  if (e == cudaSuccess) e = op_attr<float, false, false, false>(bytes);
+  return e;
 }
 
 // One V-cycle of the per-pair multigrid on level l (right side in mpl[l].b, iterate in
@@ -1262,9 +1088,7 @@ static grte_status mp_setup(grte2d_t h) {
   for (int cy = 0; cy < ncy; ++cy)
     for (int cx = 0; cx < ncx; ++cx) {
       tl_launches++, k2_mp_probe_in<<<grid_of(K * nc), kThreads, 0, st>>>(D, cx, cy, h->mp_probe);
-      tl_launches++, k2_vertex<double, false><<<grid_of(K * g.nv), kThreads, 0, st>>>(D, h->cv, UField{h->mp_probe, nc, nullptr}, h->V);
-      tl_launches++, k2_cell<double, C_MV_CORR, false><<<grid_of(K * nc), kThreads, 0, st>>>(
-          D, h->cv, h->V, UField{h->mp_probe, nc, nullptr}, h->mp_probe, h->Kr, nullptr, h->tk);
+      op_pass<double, false, false>(h, false, h->cv, h->mp_probe, nullptr, nullptr, nullptr, h->Kr, nullptr);
       tl_launches++, k2_mp_probe_out<<<grid_of(K * nc), kThreads, 0, st>>>(D, cx, cy, h->Kr, L0.cr);
     }
   for (size_t l = 0; l < h->mpl.size(); ++l) {
@@ -1295,15 +1119,6 @@ static void mp_apply(grte2d_t h, const CV<S>& cv, const S* r, S* z) {
   cudaGraphLaunch(h->mp_graph, st);
   tl_launches += h->mp_nodes;
   tl_launches++, k2_mp_out<S><<<grid_of(n), kThreads, 0, st>>>(h->D, cv, h->mpl[0].x, z);
-}
-
-static void apply_P32(grte2d_t h, bool pred, const float* r, float* z) {
-  if (!pred && h->mp_graph) {
-    mp_apply<float>(h, h->cv32, r, z);
-    return;
-  }
-  if (pred) tl_launches++, k2_prec<float, true><<<grid_of(h->D.g.nc), kThreads, 0, h->stream>>>(h->D, h->cv32, r, z);
-  else tl_launches++, k2_prec<float, false><<<grid_of(h->D.g.nc), kThreads, 0, h->stream>>>(h->D, h->cv32, r, z);
 }
 
 static void tof(grte2d_t h, const double* src, float* dst, int64_t n) {
@@ -1369,8 +1184,7 @@ static void mg_setup(grte2d_t h) {
     for (int cx = 0; cx < ncx; ++cx) {
       tl_launches++, k2_probe_in<<<grid_of(K * nc), kThreads, 0, st>>>(D, cx, cy, h->Kt);
       tl_launches++, k2_vertex<double, false><<<grid_of(K * g.nv), kThreads, 0, st>>>(D, h->cv, UField{h->Kt, nc, nullptr}, h->V);
-      tl_launches++, k2_cell<double, C_DIVK, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv, h->V, UField{h->Kt, nc, nullptr}, nullptr,
-                                                                   h->tk, nullptr, nullptr);
+      tl_launches++, k2_cell<double, C_DIVK, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv, h->V, UField{h->Kt, nc, nullptr}, h->tk);
       tl_launches++, k2_probe_out<<<grid_of(nc), kThreads, 0, st>>>(D, cx, cy, h->tk, L0.coef);
     }
   tl_launches++, mg::mg_idiag0<<<grid_of(nc), kThreads, 0, st>>>(L0);
@@ -1384,65 +1198,48 @@ static void mg_setup(grte2d_t h) {
   else tl_launches++, mg::mg_dense_inverse<2><<<1, mg::kThreadsMg, 0, st>>>(Lc, h->mg_M, h->mg_inv);
 }
 
-static void apply_P(grte2d_t h, bool pred, bool use_mg, const double* r, double* z) {
+// z = D_w P^{-1} r with the prediction's Schur multigrid
+static void apply_mg(grte2d_t h, const double* r, double* z) {
   D2& D = h->D;
   cudaStream_t st = h->stream;
-  if (!pred) {
-    if (h->mp_graph) mp_apply<double>(h, h->cv, r, z);
-    else tl_launches++, k2_prec<double, false><<<grid_of(D.g.nc), kThreads, 0, st>>>(D, h->cv, r, z);
-    return;
-  }
-  if (!use_mg) {
-    tl_launches++, k2_prec<double, true><<<grid_of(D.g.nc), kThreads, 0, st>>>(D, h->cv, r, z);
-    return;
-  }
   const int64_t K = D.g.K, nc = D.g.nc;
   tl_launches++, k2_pc_et<<<grid_of(K * nc), kThreads, 0, st>>>(D, r, h->Kt);
   tl_launches++, k2_vertex<double, false><<<grid_of(K * D.g.nv), kThreads, 0, st>>>(D, h->cv, UField{h->Kt, nc, nullptr}, h->V);
-  tl_launches++, k2_cell<double, C_DIVK, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv, h->V, UField{h->Kt, nc, nullptr}, nullptr, h->tk,
-                                                               nullptr, nullptr);
+  tl_launches++, k2_cell<double, C_DIVK, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv, h->V, UField{h->Kt, nc, nullptr}, h->tk);
   tl_launches++, k2_pc_rhs<<<grid_of(nc), kThreads, 0, st>>>(D, r, h->tk, h->mgl[0].b);
   const double* rho = mg_vcycle(h, 0);
   tl_launches++, k2_vertex<double, false><<<grid_of(K * D.g.nv), kThreads, 0, st>>>(D, h->cv, UField{nullptr, 0, rho}, h->V);
-  tl_launches++, k2_cell<double, C_DIVK, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, rho}, nullptr, h->tk,
-                                                               nullptr, nullptr);
+  tl_launches++, k2_cell<double, C_DIVK, false><<<grid_of(K * nc), kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, rho}, h->tk);
   tl_launches++, k2_pc_final<<<grid_of((K + 1) * nc), kThreads, 0, st>>>(D, r, rho, h->tk, z);
 }
 
-// One Arnoldi step in precision S: w = V_{j+1} = D_w P^{-1} M D_w^{-1} V_j (binary32: the
-// binary32 matrix and block preconditioner), orthogonalised against V_0..V_j by classical
-// Gram-Schmidt (the coefficients stay on the device; the last pass's update also gives
-// |w|^2); hc receives the Hessenberg column, hc[j+1] = |w|^2 (w not normalised).
+// One Arnoldi step in precision S: V_{j+1} = D_w P^{-1} M D_w^{-1} V_j, orthogonalised against
+// V_0..V_j by classical Gram-Schmidt (binary64: a second time where little is left of it;
+// k2_axpy), the Hessenberg column and the cycle's end decided on the device.
 template <typename S>
-static grte_status arnoldi_step(grte2d_t h, bool pred, bool mg_stage, S* V, int j, int64_t n, std::vector<double>& hc) {
+static void arnoldi_step(grte2d_t h, bool pred, bool mg_stage, const CV<S>& cv, S* V, int64_t ld, int j, int64_t n,
+                         const KStop& sp) {
   cudaStream_t st = h->stream;
-  S* vj = V + (int64_t)j * n;
-  S* w = V + (int64_t)(j + 1) * n;
-  if constexpr (sizeof(S) == 8) {
-    apply_M(h, pred, vj, h->Kr);
-    apply_P(h, pred, mg_stage, h->Kr, w);
-  } else {
-    apply_M32(h, pred, vj, h->Kr32);
-    apply_P32(h, pred, h->Kr32, w);
-  }
-  // binary32 cycles: one pass (a cycle only has to gain 1e5 and the binary64 restart
-  // corrects what the basis's loss of orthogonality costs); binary64: two passes
-  const int passes = sizeof(S) == 4 ? 1 : 2;
-  for (int pass = 0; pass < passes; ++pass) {
-    launch_mdot<S>(w, V, j + 1, n, h->part, st);
-    tl_launches++, k2_reduce_h<<<j + 1, kThreads, 0, st>>>(h->part, kDotBlocks, h->coef, h->hcol, pass == 0);
-    if (pass + 1 < passes) {
-      tl_launches++, k2_maxpy<S, false><<<kAxpyBlocks, kThreads, 0, st>>>(w, V, h->coef, j + 1, n, nullptr);
+  S* vj = V + (int64_t)j * ld;
+  S* w = V + (int64_t)(j + 1) * ld;
+  const int* stop = &h->ks->stop;
+  const double* inv = &h->ks->inv[j];
+  if (mg_stage || (!pred && h->mp_graph)) {
+    if constexpr (sizeof(S) == 8) {
+      op_pass<S, false, false>(h, pred, cv, vj, cv.iwsc, inv, nullptr, h->Kr, stop);
+      if (mg_stage) apply_mg(h, h->Kr, w);
+      else mp_apply<S>(h, cv, h->Kr, w);
     } else {
-      tl_launches++, k2_maxpy<S, true><<<kAxpyBlocks, kThreads, 0, st>>>(w, V, h->coef, j + 1, n, h->part);
-      tl_launches++, k2_reduce<<<1, kThreads, 0, st>>>(h->part, kAxpyBlocks, h->hcol + j + 1);
+      op_pass<S, false, false>(h, pred, cv, vj, cv.iwsc, inv, nullptr, h->Kr32, stop);
+      mp_apply<S>(h, cv, h->Kr32, w);
     }
+  } else {
+    op_pass<S, true, false>(h, pred, cv, vj, cv.iwsc, inv, nullptr, w, stop);
   }
-  CK2(cudaGetLastError());
-  CK2(cudaMemcpyAsync(h->pin, h->hcol, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, st));
-  CK2(cudaStreamSynchronize(st));
-  std::copy(h->pin, h->pin + j + 2, hc.begin());
-  return GRTE_OK;
+  for (int pass = 1; pass <= (sizeof(S) == 8 ? 2 : 1); ++pass) {
+    dot_launch<S>(h, w, V, ld, j + 1, n, pass);
+    tl_launches++, k2_axpy<S><<<std::min(vec_blocks(n, sizeof(S)), 2u * 152), kThreads, 0, st>>>(w, V, ld, j, n, h->part, h->ks, h->count, pass, sp, h->pin);
+  }
 }
 
 // Restarted GMRES(m) with left preconditioning on M x = b (x holds the initial
@@ -1476,35 +1273,36 @@ static grte_status gmres2(grte2d_t h, bool pred, bool mg_stage, int64_t n, int& 
   const int nblk = pred ? D.g.K + 1 : D.g.K;
   const unsigned gc = grid_of(D.g.nc);
   const int m = h->m;
+  const int64_t ld = basis_ld(n);
   double* V = h->Kbasis;
   const bool f32 = h->mixed && !mg_stage;
-  std::vector<double> H((size_t)(m + 1) * m, 0.0), g(m + 1), cs(m), sn(m), yv(m);
-  const unsigned vb = kAxpyBlocks;
+  const bool mg = mg_stage || (!pred && h->mp_graph);   // a multigrid preconditioner: several launches
   const double rtol = h->mixed ? std::max(h->opt.krylov_rtol, kMixedRtol) : h->opt.krylov_rtol;
   const double thr = rtol * std::sqrt((double)D.g.nc);
   const int maxcycles = mg_stage ? kMgStageCycles : h->opt.krylov_maxcycles;
-  grte_status s = GRTE_OK;
+  // the estimate is taken to a tenth of the threshold, the residual test to the threshold: the
+  // last cycle then leaves an error well below it (half the threshold: 5-8% fewer steps, up to
+  // ten times the error at the rounding floor)
+  const KStop sp{0.1 * thr, f32 ? kInnerReduce : 0.0, mg_stage ? 1 : 0, m};
   iters = 0;
-  auto set_scale = [&]() {
-    const double* src = pred ? h->x + (int64_t)D.g.K * D.g.nc : h->cscale;
-    tl_launches++, k2_maxabs<<<kRedBlocks, kThreads, 0, st>>>(src, D.g.nc, h->part);
-    tl_launches++, k2_weights<<<gc, kThreads, 0, st>>>(D, src, pred ? 1.0 : D.g.eps, h->part, kRedBlocks, mg_stage ? 1 : 0);
-    if (f32) {
-      tof(h, D.wsc, h->wsc32, D.g.nc);
-      tof(h, D.iwsc, h->iwsc32, D.g.nc);
-    }
-  };
-  // the true scaled residual of the unscaled x, into V_0; returns its norm
+  // the true scaled residual D_w P^{-1} (b - M x) of x into V_0; its norm
   auto residual = [&](double* beta) -> grte_status {
-    set_scale();
-    tl_launches++, k2_cellscale<<<gc, kThreads, 0, st>>>(h->x, D.wsc, nblk, D.g.nc);   // x -> y
-    apply_M(h, pred, h->x, h->Kr);
-    tl_launches++, k2_bminus<<<vb, kThreads, 0, st>>>(h->b, h->Kr, n);
-    apply_P(h, pred, mg_stage, h->Kr, V);
-    double b2 = 0.0;
-    grte_status r = mdot(h, V, V, 1, n, &b2);
-    *beta = std::sqrt(b2);
-    return r;
+    const double* src = pred ? h->x + (int64_t)D.g.K * D.g.nc : h->cscale;
+    tl_launches++, k2_maxabs<<<kRedBlocks, kThreads, 0, st>>>(src, D.g.nc, h->part, h->count, h->dots);
+    tl_launches++, k2_weights<<<gc, kThreads, 0, st>>>(D, src, pred ? 1.0 : D.g.eps, h->dots, mg_stage ? 1 : 0,
+                                                       f32 ? h->wsc32 : nullptr, h->iwsc32);
+    if (!mg) {
+      op_pass<double, true, true>(h, pred, h->cv, h->x, nullptr, nullptr, h->b, V, nullptr);
+    } else {
+      op_pass<double, false, true>(h, pred, h->cv, h->x, nullptr, nullptr, h->b, h->Kr, nullptr);
+      if (mg_stage) apply_mg(h, h->Kr, V);
+      else mp_apply<double>(h, h->cv, h->Kr, V);
+    }
+    dot_launch<double>(h, V, V, ld, 0, n, 1);
+    CK2(cudaGetLastError());
+    CK2(cudaStreamSynchronize(st));
+    *beta = std::sqrt(h->pin->r2);
+    return GRTE_OK;
   };
   // a restart cycle that did not reduce the residual 4x while it is below 1e-9 (RMS per
   // cell) has reached the rounding floor of the residual evaluation (in cold, very
@@ -1513,61 +1311,34 @@ static grte_status gmres2(grte2d_t h, bool pred, bool mg_stage, int64_t n, int& 
   double prev = INFINITY;
   for (int cycle = 0; cycle <= maxcycles; ++cycle) {
     double beta = 0.0;
-    if ((s = residual(&beta)) != GRTE_OK) return s;
+    const grte_status s = residual(&beta);
+    if (s != GRTE_OK) return s;
+    if (cycle > 0) iters += h->pin->kk;
     if (!std::isfinite(beta)) return fail2(h, GRTE_ENAN, "GMRES: non-finite residual");
     const bool floor_reached = mg_stage ? beta >= 0.25 * prev : (beta <= stall && beta >= 0.25 * prev);
     prev = beta;
     if (beta <= thr || floor_reached || cycle == maxcycles) {
       if (floor_reached) beta = 0.0;
-      tl_launches++, k2_cellscale<<<gc, kThreads, 0, st>>>(h->x, D.iwsc, nblk, D.g.nc);  // y -> x
       if (!mg_stage && !(beta <= thr)) h->host_flags |= 1 << GRTE_ENONCONV;
       return GRTE_OK;
     }
-    if (f32) tl_launches++, k2_tof<<<vb, kThreads, 0, st>>>(V, h->V32, n, 1.0 / beta);
-    else tl_launches++, k2_scale<double><<<vb, kThreads, 0, st>>>(V, 1.0 / beta, n);
-    std::fill(g.begin(), g.end(), 0.0);
-    g[0] = beta;
-    int kk = 0;
+    if (f32) tl_launches++, k2_tof<<<kAxpyBlocks, kThreads, 0, st>>>(V, h->V32, n, 1.0 / beta);
+    tl_launches++, k2_cycle_begin<<<1, 1, 0, st>>>(h->ks, beta, f32 ? 1.0 : 1.0 / beta);
+    // the multigrid preconditioners do not look at the stop flag: no step ahead of it
+    const int look = mg ? 1 : kLook;
     for (int j = 0; j < m; ++j) {
-      std::vector<double> hc(j + 2, 0.0);
-      s = f32 ? arnoldi_step<float>(h, pred, mg_stage, h->V32, j, n, hc)
-              : arnoldi_step<double>(h, pred, mg_stage, V, j, n, hc);
-      if (s != GRTE_OK) return s;
-      const double hn = std::sqrt(hc[j + 1]);
-      hc[j + 1] = hn;
-      ++iters;
-      for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * hc[i] + sn[i] * hc[i + 1];
-        hc[i + 1] = -sn[i] * hc[i] + cs[i] * hc[i + 1];
-        hc[i] = t;
+      if (j >= look) {
+        CK2(cudaEventSynchronize(h->ev[(j - look) % (kLook + 1)]));
+        if (*(volatile int*)&h->pin->stop[j - look]) break;
       }
-      const double rr = std::hypot(hc[j], hc[j + 1]);
-      cs[j] = rr > 0.0 ? hc[j] / rr : 1.0;
-      sn[j] = rr > 0.0 ? hc[j + 1] / rr : 0.0;
-      hc[j] = rr;
-      g[j + 1] = -sn[j] * g[j];
-      g[j] = cs[j] * g[j];
-      for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hc[i];
-      kk = j + 1;
-      if (hn > 0.0) {
-        if (f32) tl_launches++, k2_scale<float><<<vb, kThreads, 0, st>>>(h->V32 + (int64_t)(j + 1) * n, 1.0 / hn, n);
-        else tl_launches++, k2_scale<double><<<vb, kThreads, 0, st>>>(V + (int64_t)(j + 1) * n, 1.0 / hn, n);
-      }
-      const double gj = std::fabs(g[j + 1]);
-      if (gj <= 0.5 * thr || hn == 0.0) break;
-      if (f32 && gj <= kInnerReduce * beta) break;
-      if (mg_stage && j >= 4 && gj <= 1e-6 * beta && gj > 0.5 * std::fabs(g[j - 3])) break;
+      if (f32) arnoldi_step<float>(h, pred, mg_stage, h->cv32, h->V32, ld, j, n, sp);
+      else arnoldi_step<double>(h, pred, mg_stage, h->cv, V, ld, j, n, sp);
+      CK2(cudaEventRecord(h->ev[j % (kLook + 1)], st));
     }
-    for (int i = kk - 1; i >= 0; --i) {
-      double t = g[i];
-      for (int l = i + 1; l < kk; ++l) t -= H[(size_t)i * m + l] * yv[l];
-      yv[i] = t / H[(size_t)i * m + i];
-    }
-    CK2(cudaMemcpyAsync(h->coef, yv.data(), sizeof(double) * kk, cudaMemcpyHostToDevice, st));
-    if (f32) tl_launches++, k2_update<float><<<vb, kThreads, 0, st>>>(h->x, h->V32, h->coef, kk, n);
-    else tl_launches++, k2_update<double><<<vb, kThreads, 0, st>>>(h->x, V, h->coef, kk, n);
-    tl_launches++, k2_cellscale<<<gc, kThreads, 0, st>>>(h->x, D.iwsc, nblk, D.g.nc);    // y -> x
-    CK2(cudaStreamSynchronize(st));
+    tl_launches++, k2_solve_y<<<1, 32, 0, st>>>(h->ks);
+    const dim3 ug(gc, (unsigned)nblk);
+    if (f32) tl_launches++, k2_update<float><<<ug, kThreads, 0, st>>>(h->x, h->V32, ld, D.g.nc, D.iwsc, h->ks);
+    else tl_launches++, k2_update<double><<<ug, kThreads, 0, st>>>(h->x, V, ld, D.g.nc, D.iwsc, h->ks);
     CK2(cudaGetLastError());
   }
   return GRTE_OK;
@@ -1587,7 +1358,7 @@ static grte_status step2(grte2d_t h) {
   tl_launches++, k2_vcoef<<<gv, kThreads, 0, st>>>(D);
   tl_launches++, k2_rho<<<gc, kThreads, 0, st>>>(D, D.E, D.rho_n);
   tl_launches++, k2_vertex<double, true><<<gvk, kThreads, 0, st>>>(D, h->cv, UField{nullptr, 0, nullptr}, h->V);
-  tl_launches++, k2_cell<double, C_DIVK, true><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, nullptr}, nullptr, h->phi, nullptr, nullptr);
+  tl_launches++, k2_cell<double, C_DIVK, true><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, nullptr}, h->phi);
   tl_launches++, k2_rhs_pred<<<gc, kThreads, 0, st>>>(D, h->phi, h->b, h->x);
   tl_launches++, k2_gdiag<<<gc, kThreads, 0, st>>>(D, h->cv);
   mirror_coefficients(h);
@@ -1620,9 +1391,9 @@ static grte_status step2(grte2d_t h) {
     tl_launches++, k2_fdiv_corr<<<gck, kThreads, 0, st>>>(D, h->cv, h->V, Vp, UField{h->Es, nc, nullptr}, h->tk);
   } else {
     tl_launches++, k2_vertex<double, true><<<gvk, kThreads, 0, st>>>(D, h->cv, UField{h->Es, nc, nullptr}, h->V);
-    tl_launches++, k2_cell<double, C_FDIV, true><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{h->Es, nc, nullptr}, nullptr, nullptr, nullptr, h->tk);
+    tl_launches++, k2_cell<double, C_FDIV, true><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{h->Es, nc, nullptr}, h->tk);
   }
-  tl_launches++, k2_cellsum<double, C_FDIV><<<gc, kThreads, 0, st>>>(D, h->cv, h->tk, nullptr, D.Fdiv, nullptr);
+  tl_launches++, k2_cellsum<<<gc, kThreads, 0, st>>>(D, h->tk, D.Fdiv);
   if (D.use_guess || D.log_samples) tl_launches++, k2_newton_feat<<<gc, kThreads, 0, st>>>(D);
   if (D.use_guess) {
     tl_launches++;   // the network's guess: one kernel
@@ -1635,9 +1406,9 @@ static grte_status step2(grte2d_t h) {
   tl_launches++, k2_vcoef<<<gv, kThreads, 0, st>>>(D);
   tl_launches++, k2_acU<<<gc, kThreads, 0, st>>>(D);
   tl_launches++, k2_vertex<double, true><<<gvk, kThreads, 0, st>>>(D, h->cv, UField{nullptr, 0, nullptr}, h->V);
-  tl_launches++, k2_cell<double, C_DIVK, true><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, nullptr}, nullptr, h->phi, nullptr, nullptr);
+  tl_launches++, k2_cell<double, C_DIVK, true><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, nullptr}, h->phi);
   tl_launches++, k2_vertex<double, false><<<gvk, kThreads, 0, st>>>(D, h->cv, UField{nullptr, 0, D.acU}, h->V);
-  tl_launches++, k2_cell<double, C_DIVK, false><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, D.acU}, nullptr, h->GU, nullptr, nullptr);
+  tl_launches++, k2_cell<double, C_DIVK, false><<<gck, kThreads, 0, st>>>(D, h->cv, h->V, UField{nullptr, 0, D.acU}, h->GU);
   tl_launches++, k2_rhs_corr<<<gc, kThreads, 0, st>>>(D, h->GU, h->phi, h->b, h->x);
   tl_launches++, k2_corrscale<<<gc, kThreads, 0, st>>>(D, h->cscale);
   tl_launches++, k2_gdiag<<<gc, kThreads, 0, st>>>(D, h->cv);
@@ -1664,6 +1435,7 @@ void grte2d_destroy(grte2d_t h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->mp_graph) cudaGraphExecDestroy(h->mp_graph);
   if (h->pin) cudaFreeHost(h->pin);
+  for (cudaEvent_t e : h->ev) if (e) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
@@ -1751,13 +1523,15 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
             alloc2(h, &D.wsc, nc) && alloc2(h, &D.iwsc, nc) && alloc2(h, &D.gd, K * nc) && alloc2(h, &D.gdi, K * nc) && alloc2(h, &D.pdi, nc) &&
             alloc2(h, &h->V, K * nv) && alloc2(h, &h->phi, K * nc) && alloc2(h, &h->GU, K * nc) &&
             alloc2(h, &h->Es, K * nc) && alloc2(h, &h->b, nz) && alloc2(h, &h->x, nz) && alloc2(h, &h->Kr, nz) &&
-            alloc2(h, &h->Kt, nz) && alloc2(h, &h->Kbasis, (int64_t)(h->m + 1) * nz) &&
+            alloc2(h, &h->Kt, nz) && alloc2(h, &h->Kbasis, (int64_t)(h->m + 1) * basis_ld(nz)) &&
             alloc2(h, &h->part, (int64_t)kAxpyBlocks * (kMaxRestart2 + 1)) && alloc2(h, &h->dots, kMaxRestart2 + 1) &&
-            alloc2(h, &h->coef, kMaxRestart2 + 1) && alloc2(h, &h->cscale, nc) &&
-            alloc2(h, &h->hcol, kMaxRestart2 + 2) && alloc2(h, &h->tk, K * nc);
+            alloc2(h, &h->cscale, nc) && alloc2(h, &h->tk, K * nc) && alloc2(h, &h->ks, 1) && alloc2(h, &h->count, 1);
   if (!ok) return fail2(h, GRTE_ENOMEM, "cudaMalloc failed");
-  if (cudaMallocHost(&h->pin, sizeof(double) * (kMaxRestart2 + 2)) != cudaSuccess)
-    return fail2(h, GRTE_ENOMEM, "cudaMallocHost failed");
+  if (cudaMallocHost(&h->pin, sizeof(KPin)) != cudaSuccess) return fail2(h, GRTE_ENOMEM, "cudaMallocHost failed");
+  CK2(cudaMemset(h->ks, 0, sizeof(KState)));
+  CK2(cudaMemset(h->count, 0, sizeof(unsigned)));
+  for (cudaEvent_t& e : h->ev) CK2(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  CK2(op_attrs());
   if (h->opt.prec2d & ~(GRTE_PREC2D_MULTIGRID | GRTE_PREC2D_CORR_MG))
     return fail2(h, GRTE_EINVAL, "prec2d: a set of GRTE_PREC2D_MULTIGRID and GRTE_PREC2D_CORR_MG");
   if (h->opt.prec2d & GRTE_PREC2D_CORR_MG) {
@@ -1804,13 +1578,11 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
                      g.h2x, g.h2y, g.te};
   if (h->opt.precision == GRTE_MIXED) {
     h->mixed = true;
-    const int64_t nvk = K * nv;
     bool okf = alloc2(h, &h->mu32, K) && alloc2(h, &h->eta32, K) && alloc2(h, &h->w32, K) &&
                alloc2(h, &h->kc32, nc) && alloc2(h, &h->A32, nc) && alloc2(h, &h->alpha32, nc) &&
                alloc2(h, &h->dv32, nv) && alloc2(h, &h->gd32, K * nc) && alloc2(h, &h->gdi32, K * nc) &&
                alloc2(h, &h->pdi32, nc) && alloc2(h, &h->wsc32, nc) && alloc2(h, &h->iwsc32, nc) &&
-               alloc2(h, &h->V32, (int64_t)(h->m + 1) * nz) && alloc2(h, &h->Kr32, nz) &&
-               alloc2(h, &h->Vv32, nvk) && alloc2(h, &h->tk32, K * nc);
+               alloc2(h, &h->V32, (int64_t)(h->m + 1) * basis_ld(nz)) && alloc2(h, &h->Kr32, nz);
     if (!okf) return fail2(h, GRTE_ENOMEM, "cudaMalloc binary32 buffers");
     std::vector<float> f(K);
     for (int64_t k = 0; k < K; ++k) f[k] = (float)h->hmu[k];
@@ -1842,7 +1614,7 @@ grte_status grte2d_set_state(grte2d_t h, const double* T, const double* E, const
   D2& D = h->D;
   cudaStream_t st = h->stream;
   CK2(cudaMemcpyAsync(D.T, T, sizeof(double) * nc, cudaMemcpyHostToDevice, st));
-  k_fourth_power<<<grid_of(nc), kThreads, 0, st>>>(D.T, D.U, nc);
+  k2_fourth_power<<<grid_of(nc), kThreads, 0, st>>>(D);
   if (E) {
     // the arrays in the host's layout pass through the Krylov basis, free between solves
     CK2(cudaMemcpyAsync(h->Kbasis, E, sizeof(double) * K * nc, cudaMemcpyHostToDevice, st));
@@ -1862,9 +1634,9 @@ grte_status grte2d_set_state(grte2d_t h, const double* T, const double* E, const
 }
 
 static grte_status status2(grte2d_t h) {
-  CK2(cudaMemcpyAsync(h->pin, h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CK2(cudaMemcpyAsync(&h->pin->status, h->D.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CK2(cudaStreamSynchronize(h->stream));
-  int s = *(const int*)h->pin;
+  int s = h->pin->status;
   s |= h->host_flags;
   h->stats.status_flags = s;
   for (int code : {GRTE_ENAN, GRTE_ENONCONV, GRTE_ENEGATIVE, GRTE_ETIMEOUT})
