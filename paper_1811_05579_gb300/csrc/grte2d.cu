@@ -597,19 +597,36 @@ __global__ void k2_pc_final(D2 D, const double* __restrict__ r, const double* __
   z[t] = t < ne ? D.wsc[c] * D.gdi[t] * (r[t] - D.alpha[c] * rho[c] - tk[t]) : D.wsc[c] * rho[c];
 }
 
+// 1/x in binary64 from a binary32 seed and two Newton-Raphson steps (relative error at binary64
+// rounding; 4 operations instead of the divide sequence); outside the binary32 range the plain
+// division.
+__device__ __forceinline__ double recip(double x) {
+  if (!(fabs(x) > 1e-30 && fabs(x) < 1e30)) return 1.0 / x;
+  double y = (double)__frcp_rn((float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
 // gd[k][c] = diagonal of G_k at cell c (for the preconditioner), at the current coefficients
 // and the reciprocals the preconditioner needs: gdi = 1/(A + g_k) and, per cell, the
-// inverse of the arrow block's rho pivot alpha + sum_k w_k g_k (A - alpha)/(A + g_k).
+// arrow matrix's inverse rho pivot.  Away from the walls g_k = kappa [a^2 (d00 + d11) +
+// b^2 (d10 + d01)], a, b = mu/(2dx) +- eta/(2dy) and d the cell's vertex coefficients.
 __global__ void k2_gdiag(D2 D, CV<double> cv) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const G2& g = D.g;
   if (c >= g.nc) return;
   const int p = (int)(c % g.Nx), q = (int)(c / g.Nx);
-  const double A = D.A[c], al = D.alpha[c];
+  const double A = D.A[c], al = D.alpha[c], kc = D.kc[c];
+  const bool wall = (g.bcx == GRTE_BC_INFLOW && (p == 0 || p == g.Nx - 1)) ||
+                    (g.bcy == GRTE_BC_INFLOW && (q == 0 || q == g.Ny - 1));
+  const int64_t v = (int64_t)q * (g.Nx + 1) + p;
+  const double da = kc * (D.dv[v] + D.dv[v + g.Nx + 2]), db = kc * (D.dv[v + 1] + D.dv[v + g.Nx + 1]);
   double den = al;
   for (int k = 0; k < g.K; ++k) {
     const int64_t o = (int64_t)k * g.nc + c;
-    const double gk = gdiag(D, cv, k, p, q), inv = 1.0 / (A + gk);
+    const double mx = D.mu[k] * g.h2x, ey = D.eta[k] * g.h2y, a = mx + ey, b = mx - ey;
+    const double gk = wall ? gdiag(D, cv, k, p, q) : fma(a * a, da, b * b * db);
+    const double inv = recip(A + gk);
     D.gd[o] = gk;
     D.gdi[o] = inv;
     den += D.w[k] * gk * (A - al) * inv;
@@ -632,15 +649,15 @@ __global__ void k2_rhs_pred(D2 D, const double* __restrict__ phi, double* __rest
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const G2& g = D.g;
   if (c >= g.nc) return;
-  const double cdt = g.c * g.dt, sac = D.s[c] * g.a * g.c * D.U[c], kc = D.kc[c], rn = D.rho_n[c];
+  const double sac = D.s[c] * g.a * g.c * D.U[c], kcd = D.kc[c] / (g.c * g.dt), rn = D.rho_n[c];
   double ps = 0.0;
   for (int k = 0; k < g.K; ++k) {
     const int64_t o = (int64_t)k * g.nc + c;
-    b[o] = kc * D.E[o] / cdt + sac - phi[o];
+    b[o] = kcd * D.E[o] + sac - phi[o];
     x[o] = D.E[o] - rn;
     ps += D.w[k] * phi[o];
   }
-  b[(int64_t)g.K * g.nc + c] = kc * rn / cdt + sac - ps;
+  b[(int64_t)g.K * g.nc + c] = kcd * rn + sac - ps;
   x[(int64_t)g.K * g.nc + c] = rn;
 }
 
@@ -670,10 +687,10 @@ __global__ void k2_rhs_corr(D2 D, const double* __restrict__ GU, const double* _
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const G2& g = D.g;
   if (c >= g.nc) return;
-  const double cdt = g.c * g.dt, kc = D.kc[c], acU = D.acU[c];
+  const double kcd = D.kc[c] / (g.c * g.dt), acU = D.acU[c], ieps = 1.0 / g.eps;
   for (int k = 0; k < g.K; ++k) {
     const int64_t o = (int64_t)k * g.nc + c;
-    b[o] = (kc * (D.E[o] - acU) / cdt - GU[o] - phi[o]) / g.eps;
+    b[o] = (kcd * (D.E[o] - acU) - GU[o] - phi[o]) * ieps;
     x[o] = 0.0;
   }
 }
@@ -982,22 +999,33 @@ static void op_pass(grte2d_t h, bool pred, const CV<S>& cv, const S* z, const S*
   else go(std::false_type{});
 }
 
-// The vector kernels' blocks for n values: four 16-byte groups per thread, at most four blocks
-// per SM.
-static unsigned vec_blocks(int64_t n, size_t es) {
-  const int64_t groups = n / (int64_t)(16 / es) + 1;
-  return (unsigned)std::min<int64_t>((groups + 4 * kThreads - 1) / (4 * kThreads), kVecBlocks);
+// The vector kernels: one 16-byte group per thread up to a full wave of blocks; the chunk
+// template by the number of vectors, so that few vectors leave registers for more blocks.
+template <typename S>
+static unsigned vec_blocks(int64_t n, int per_sm) {
+  const int64_t groups = n / (int64_t)(16 / sizeof(S)) + 1;
+  return (unsigned)std::min<int64_t>((groups + kThreads - 1) / kThreads, per_sm * 152);
 }
 template <typename S>
 static void dot_launch(grte2d_t h, const S* w, const S* V, int64_t ld, int nv, int64_t n, int pass) {
-  const unsigned nb = vec_blocks(n, sizeof(S));
   auto go = [&](auto C, int per_sm) {
-    k2_dot<S, decltype(C)::value><<<std::min<unsigned>(nb, per_sm * 152), kThreads, 0, h->stream>>>(
+    k2_dot<S, decltype(C)::value><<<vec_blocks<S>(n, per_sm), kThreads, 0, h->stream>>>(
         w, V, ld, nv, n, h->part, h->ks, h->count, pass, h->pin);
     tl_launches++;
   };
   if (nv <= 3) go(std::integral_constant<int, 4>{}, 4);
   else if (nv <= 7) go(std::integral_constant<int, 8>{}, 3);
+  else go(std::integral_constant<int, 16>{}, 2);
+}
+template <typename S>
+static void axpy_launch(grte2d_t h, S* w, const S* V, int64_t ld, int j, int64_t n, int pass, const KStop& sp) {
+  auto go = [&](auto C, int per_sm) {
+    k2_axpy<S, decltype(C)::value><<<vec_blocks<S>(n, per_sm), kThreads, 0, h->stream>>>(
+        w, V, ld, j, n, h->part, h->ks, h->count, pass, sp, h->pin);
+    tl_launches++;
+  };
+  if (j < 4) go(std::integral_constant<int, 4>{}, 4);
+  else if (j < 8) go(std::integral_constant<int, 8>{}, 3);
   else go(std::integral_constant<int, 16>{}, 2);
 }
 
@@ -1219,7 +1247,6 @@ static void apply_mg(grte2d_t h, const double* r, double* z) {
 template <typename S>
 static void arnoldi_step(grte2d_t h, bool pred, bool mg_stage, const CV<S>& cv, S* V, int64_t ld, int j, int64_t n,
                          const KStop& sp) {
-  cudaStream_t st = h->stream;
   S* vj = V + (int64_t)j * ld;
   S* w = V + (int64_t)(j + 1) * ld;
   const int* stop = &h->ks->stop;
@@ -1238,7 +1265,7 @@ static void arnoldi_step(grte2d_t h, bool pred, bool mg_stage, const CV<S>& cv, 
   }
   for (int pass = 1; pass <= (sizeof(S) == 8 ? 2 : 1); ++pass) {
     dot_launch<S>(h, w, V, ld, j + 1, n, pass);
-    tl_launches++, k2_axpy<S><<<std::min(vec_blocks(n, sizeof(S)), 2u * 152), kThreads, 0, st>>>(w, V, ld, j, n, h->part, h->ks, h->count, pass, sp, h->pin);
+    axpy_launch<S>(h, w, V, ld, j, n, pass, sp);
   }
 }
 
@@ -1280,10 +1307,10 @@ static grte_status gmres2(grte2d_t h, bool pred, bool mg_stage, int64_t n, int& 
   const double rtol = h->mixed ? std::max(h->opt.krylov_rtol, kMixedRtol) : h->opt.krylov_rtol;
   const double thr = rtol * std::sqrt((double)D.g.nc);
   const int maxcycles = mg_stage ? kMgStageCycles : h->opt.krylov_maxcycles;
-  // the estimate is taken to a tenth of the threshold, the residual test to the threshold: the
+  // binary64: the estimate is taken to a tenth of the threshold, the residual test to it: the
   // last cycle then leaves an error well below it (half the threshold: 5-8% fewer steps, up to
   // ten times the error at the rounding floor)
-  const KStop sp{0.1 * thr, f32 ? kInnerReduce : 0.0, mg_stage ? 1 : 0, m};
+  const KStop sp{(f32 ? 0.5 : 0.1) * thr, f32 ? kInnerReduce : 0.0, mg_stage ? 1 : 0, m};
   iters = 0;
   // the true scaled residual D_w P^{-1} (b - M x) of x into V_0; its norm
   auto residual = [&](double* beta) -> grte_status {

@@ -54,15 +54,17 @@ struct KPin {
 // their weighted sum is complete and the preconditioner can be applied.  In terms of
 // a = mu/(2dx) + eta/(2dy), b = mu/(2dx) - eta/(2dy) both stencils are four operations:
 //   D_k u = a (u11 - u00) + b (u10 - u01)   (and the same over the vertices of a cell).
+// A thread keeps to one cell, its lower left vertex, and (the first threads) one halo cell and
+// one vertex of the tile's upper or right edge, so that every index is formed once per block.
 // G groups of threads share the pairs of a tile, each with its own barrier.
-// Bound: binary64 the FP64 pipe (about 23 operations per cell and pair; the separate vertex,
+// Bound: binary64 the FP64 pipe (about 22 operations per cell and pair; the separate vertex,
 // cell, sum and preconditioner kernels took about 60), binary32 issue and L1; the vectors are
-// read and written once.  512^2 cells, 20 pairs: 49 us (prediction) and 36 us (correction) in
-// binary32, 398 and 325 us in binary64, against 127 and 108, and 560 and 480, of the separate
-// kernels; 61 x 47 in binary64 19 and 15 us against 53 and 34.
+// read and written once.  512^2 cells, 20 pairs, prediction and correction: 49 and 34 us in
+// binary32, 347 and 263 us in binary64 (the separate kernels 127 and 108, 560 and 480); 192^2 in
+// binary64 56 and 52 us (105 and 101), 61 x 47 15 and 12 us (53 and 34).
 template <typename S>
 __host__ __device__ constexpr size_t op_smem(int K, int TX, int TY, int G, bool prec) {
-  return sizeof(S) * ((size_t)(TY + 2) * (TX + 2) * (2 + G) + (size_t)(TY + 1) * (TX + 1) * G + 5 * (size_t)K +
+  return sizeof(S) * ((size_t)(TY + 2) * (TX + 2) * G + (size_t)(TY + 1) * (TX + 1) * G + 7 * (size_t)K +
                       (size_t)2 * TX * TY * G + (prec ? (size_t)K * TX * TY : 0));
 }
 
@@ -75,24 +77,28 @@ __device__ __forceinline__ void group_sync(int gq) {
   else asm volatile("bar.sync %0, %1;" ::"r"(gq + 1), "n"(NT) : "memory");
 }
 
+// Blocks per SM that the registers have to leave room for: binary32 32 x 8 tiles live on many
+// warps in flight, the 32 x 4 tiles of four groups must all be resident at once (a second,
+// partial wave would double their time).
+template <typename S, int TX, int TY, int G>
+constexpr int op_min_blocks() { return TX == 8 ? 1 : G > 1 ? 2 : sizeof(S) == 4 ? 5 : 3; }
+
 template <typename S, bool PRED, bool PREC, bool RES, int TX, int TY, int G>
-__global__ void __launch_bounds__(TX * TY * G) k2_op(D2 D, CV<S> cv, const S* __restrict__ z,
-                                                     const S* __restrict__ sc, const double* __restrict__ inv,
-                                                     const S* __restrict__ b, S* __restrict__ out,
-                                                     const int* __restrict__ stop) {
+__global__ void __launch_bounds__(TX * TY * G, op_min_blocks<S, TX, TY, G>())
+    k2_op(D2 D, CV<S> cv, const S* __restrict__ z, const S* __restrict__ sc, const double* __restrict__ inv,
+          const S* __restrict__ b, S* __restrict__ out, const int* __restrict__ stop) {
   if (stop && *stop) return;
   constexpr int NT = TX * TY;                       // threads of a group = cells of the tile
   constexpr int LC = TX + 2, LV = TX + 1;           // row lengths of the cell and vertex tiles
   constexpr int NC = (TY + 2) * LC, NV = (TY + 1) * LV;
-  constexpr int RC = (NC + NT - 1) / NT, RV = (NV + NT - 1) / NT;
+  constexpr int NH = 2 * LC + 2 * TY, NE = LV + TY; // halo cells; vertices of the upper and right edge
   static_assert(NT % 32 == 0 && G < 16, "a group is whole warps, one hardware barrier each");
+  static_assert(NH <= NT && NE <= NT, "one halo cell and one edge vertex per thread");
   extern __shared__ __align__(16) unsigned char op_raw[];
   const G2& g = D.g;
-  const int K = g.K, nc = (int)g.nc;
+  const int K = g.K, nc = (int)g.nc;                // K nc < 2^31 (checked at creation)
   const int tid = threadIdx.x % NT, gq = threadIdx.x / NT, lx = tid % TX, ly = tid / TX;
   S* p = reinterpret_cast<S*>(op_raw);
-  S* const sf = p;   p += NC;                       // scale of the tile's cells
-  S* const su = p;   p += NC;                       // scaled rho part
   S* const tu = p + gq * NC;   p += G * NC;         // u of the group's pair
   S* const tv = p + gq * NV;   p += G * NV;         // its vertex values
   S* const ka = p;   p += K;
@@ -100,6 +106,8 @@ __global__ void __launch_bounds__(TX * TY * G) k2_op(D2 D, CV<S> cv, const S* __
   S* const kmu = p;  p += K;
   S* const keta = p; p += K;
   S* const kw = p;   p += K;
+  S* const kex = p;  p += K;                        // |mu| (2/eps)/dx, |eta| (2/eps)/dy: a wall
+  S* const key = p;  p += K;                        // side's coefficient of E_cell (cell_sides)
   S* const red = p;  p += 2 * NT * G;
   S* const rows = p;                                // [k][cell of the tile]
   const int p0 = blockIdx.x * TX, q0 = blockIdx.y * TY;
@@ -111,103 +119,124 @@ __global__ void __launch_bounds__(TX * TY * G) k2_op(D2 D, CV<S> cv, const S* __
     kmu[k] = mu;
     keta[k] = eta;
     kw[k] = cv.w[k];
+    kex[k] = fabs(mu) * (cv.te * S(2) * cv.h2x);
+    key[k] = fabs(eta) * (cv.te * S(2) * cv.h2y);
   }
-  // this thread's cells of the haloed tile (the same for every pair) and its vertices
-  int cc[RC];
-#pragma unroll
-  for (int r = 0; r < RC; ++r) {
-    const int e = tid + r * NT;
-    const int c = e < NC ? cell_of(g, p0 - 1 + e % LC, q0 - 1 + e / LC) : -1;
-    cc[r] = c;
-    if (e < NC && gq == 0) {
-      const S f = c >= 0 ? (sc ? sc[c] * iv : iv) : S(0);
-      sf[e] = f;
-      su[e] = PRED && c >= 0 ? z[(int64_t)K * nc + c] * f : S(0);
-    }
-  }
-  S dv[RV];
-  int vk[RV];      // 0: node equation, 2/3: x/y wall, else nothing to form
-#pragma unroll
-  for (int r = 0; r < RV; ++r) {
-    const int e = tid + r * NT, i = p0 + e % LV, j = q0 + e / LV;
-    const bool in = e < NV && i <= g.Nx && j <= g.Ny;
-    vk[r] = in ? vkind(g, i, j) : -1;
-    dv[r] = in ? cv.dv[(int64_t)j * (g.Nx + 1) + i] : S(0);
-  }
+  // the thread's cell: scale and scaled rho part, then what its row needs
   const int pc = p0 + lx, qc = q0 + ly;
   const bool live = pc < g.Nx && qc < g.Ny;
-  const int c = live ? qc * g.Nx + pc : 0;
-  const bool wall = live && ((g.bcx == GRTE_BC_INFLOW && (pc == 0 || pc == g.Nx - 1)) ||
-                             (g.bcy == GRTE_BC_INFLOW && (qc == 0 || qc == g.Ny - 1)));
+  const int oc = (ly + 1) * LC + lx + 1;            // in the tile
+  // (past the domain: a halo cell of a live one, or on a periodic axis its image)
+  const int c = live ? qc * g.Nx + pc : cell_of(g, pc, qc);
+  const S fc = c >= 0 ? (sc ? sc[c] * iv : iv) : S(0);
+  const S rc = PRED && c >= 0 ? z[K * nc + c] * fc : S(0);
   const S A = live ? cv.A[c] : S(0), kc = live ? cv.kc[c] : S(0), al = PRED && live ? cv.alpha[c] : S(0);
-  const S ws = PREC && live ? cv.wsc[c] : S(1);
+  const S ws = PREC && live ? cv.wsc[c] : S(1), arc = al * rc;
+  const bool xw = g.bcx == GRTE_BC_INFLOW, yw = g.bcy == GRTE_BC_INFLOW;
+  // side weights of the general form (cell_sides), for tiles that touch an inflow wall
+  const bool wl = xw && pc == 0, wr = xw && pc == g.Nx - 1, wb = yw && qc == 0, wt = yw && qc == g.Ny - 1;
+  const S cL = cv.h2x * (wl ? S(0) : wr ? S(-2) : S(-1)), cR = cv.h2x * (wr ? S(0) : wl ? S(2) : S(1));
+  const S cB = cv.h2y * (wb ? S(0) : wt ? S(-2) : S(-1)), cT = cv.h2y * (wt ? S(0) : wb ? S(2) : S(1));
+  // its halo cell: lower row, upper row, left and right columns
+  int hc = -1, ho = 0;
+  S hf = S(0), hu = S(0);
+  if (tid < NH) {
+    const int hx = tid < 2 * LC ? tid % LC : (tid - 2 * LC) % 2 * (TX + 1);
+    const int hy = tid < LC ? 0 : tid < 2 * LC ? TY + 1 : 1 + (tid - 2 * LC) / 2;
+    ho = hy * LC + hx;
+    hc = cell_of(g, p0 - 1 + hx, q0 - 1 + hy);
+    if (hc >= 0) {
+      hf = sc ? sc[hc] * iv : iv;
+      if (PRED) hu = z[K * nc + hc] * hf;
+    }
+  }
+  // its vertices: the cell's lower left one, and one of the upper row or right column
+  const int ov = ly * LV + lx, ex = tid < LV ? tid : TX, ey = tid < LV ? TY : tid - LV;
+  auto vertex_kind = [&](int i, int j) { return i <= g.Nx && j <= g.Ny ? vkind(g, i, j) : -1; };
+  auto vertex_d = [&](int i, int j) { return i <= g.Nx && j <= g.Ny ? cv.dv[(int64_t)j * (g.Nx + 1) + i] : S(0); };
+  const S d0 = vertex_d(pc, qc), d1 = tid < NE ? vertex_d(p0 + ex, q0 + ey) : S(0);
+  const int k0 = vertex_kind(pc, qc), k1 = tid < NE ? vertex_kind(p0 + ex, q0 + ey) : -1;
+  // The tile's inflow-wall vertices (x walls: TY + 1 each, y walls: TX + 1 each; corners enter no
+  // cell), one per thread from the first on: one or two warps take the wall expression instead
+  // of every warp that has a wall cell.  The vertex, its wall and its inner vertex's coefficient:
+  constexpr int NW = 2 * (LV + TY + 1);
+  int wk = 0, wvx = 0, wvy = 0;
+  S wd = S(0);
+  for (int t = tid; t < NW && wk == 0; t += NT) {
+    const bool x = t < 2 * (TY + 1);
+    const int u = x ? t : t - 2 * (TY + 1), len = x ? TY + 1 : LV, r = u % len;
+    const bool lo = u < len;
+    const int i = x ? (lo ? 0 : g.Nx) : p0 + r, j = x ? q0 + r : (lo ? 0 : g.Ny);
+    if (i < p0 || i > p0 + TX || j < q0 || j > q0 + TY || i > g.Nx || j > g.Ny) continue;
+    if (vkind(g, i, j) != (x ? 2 : 3)) continue;
+    wk = x ? (lo ? 1 : 2) : (lo ? 3 : 4);
+    wvx = i - p0;
+    wvy = j - q0;
+    wd = cv.dv[(int64_t)(j + (x ? 0 : lo ? 1 : -1)) * (g.Nx + 1) + i + (x ? (lo ? 1 : -1) : 0)];
+  }
+  // a tile away from the inflow walls has node equations only (uniform over the block)
+  const bool edge = (xw && (p0 == 0 || p0 + TX >= g.Nx)) || (yw && (q0 == 0 || q0 + TY >= g.Ny));
+  if (edge)
+    for (int e = tid; e < NV; e += NT) tv[e] = S(0);   // (corners, and past the grid)
   __syncthreads();
-  const int oc = (ly + 1) * LC + lx + 1;            // the thread's cell in the tile
-  const S fc = sf[oc], rc = su[oc], arc = al * rc;
   // sum w_k kappa S_k, and the preconditioner's sum w_k g_k r_k/(A+g_k) (apart: at inflow walls
   // the first cancels against the right-hand side to a 1/eps-th of its terms)
   S st = S(0), sp = S(0);
   // the next pair's values are loaded while the current one is worked on
-  S nx[RC], nz = S(0), nb = S(0), ngd = S(0), ngi = S(0);
+  S nz = S(0), nh = S(0), nb = S(0), ngd = S(0), ngi = S(0);
   auto fetch = [&](int k) {
-#pragma unroll
-    for (int r = 0; r < RC; ++r) nx[r] = k < K && cc[r] >= 0 ? z[(int64_t)k * nc + cc[r]] : S(0);
-    if (k < K && live) {
-      const int64_t o = (int64_t)k * nc + c;
-      nz = z[o];
-      if (RES) nb = b[o];
-      if (PREC) ngi = cv.gdi[o];
-      if (PREC && PRED) ngd = cv.gd[o];
+    if (k >= K) return;
+    const int o = k * nc;
+    if (c >= 0) nz = z[o + c];
+    if (hc >= 0) nh = z[o + hc];
+    if (live) {
+      if (RES) nb = b[o + c];
+      if (PREC) ngi = cv.gdi[o + c];
+      if (PREC && PRED) ngd = cv.gd[o + c];
     }
   };
   fetch(gq);
   for (int k = gq; k < K; k += G) {
-#pragma unroll
-    for (int r = 0; r < RC; ++r) {
-      const int e = tid + r * NT;
-      if (e < NC) tu[e] = PRED ? fma(nx[r], sf[e], su[e]) : nx[r] * sf[e];
-    }
-    const S ec = nz * fc, bk = nb, gdk = ngd, gik = ngi;
+    const S ec = nz * fc, uc = PRED ? fma(nz, fc, rc) : ec, bk = nb, gdk = ngd, gik = ngi;
+    tu[oc] = uc;
+    // (not over another thread's own cell: the halo is the ring around the tile)
+    if (tid < NH) tu[ho] = PRED ? fma(nh, hf, hu) : nh * hf;
     group_sync<NT, G>(gq);
     fetch(k + G);
     const S a = ka[k], bb = kb[k];
     auto node = [&](int o, S d) {   // O at the vertex whose lower left cell is at o
       return -d * fma(a, tu[o + LC + 1] - tu[o], bb * (tu[o + 1] - tu[o + LC]));
     };
-#pragma unroll
-    for (int r = 0; r < RV; ++r) {
-      const int e = tid + r * NT, vx = e % LV, vy = e / LV, o = vy * LC + vx;
-      if (e >= NV) continue;
-      S v = S(0);
-      if (vk[r] == 0) {
-        v = node(o, dv[r]);
-      } else if (vk[r] == 2 || vk[r] == 3) {
+    S v00 = S(0);
+    if (!edge) {
+      v00 = node(oc - LC - 1, d0);
+      tv[ov] = v00;
+      if (tid < NE) tv[ey * LV + ex] = node(ey * LC + ex, d1);
+    } else {
+      if (k0 == 0) tv[ov] = node(oc - LC - 1, d0);
+      if (tid < NE && k1 == 0) tv[ey * LV + ex] = node(ey * LC + ex, d1);
+      if (wk != 0) {
         // Eq. bc-pre along the wall's normal with E the mean of the two wall cells
-        const int i = p0 + vx, j = q0 + vy;
-        const bool xw = vk[r] == 2, lo = xw ? i == 0 : j == 0;
-        const S comp = xw ? kmu[k] : keta[k];
-        const S sg = (lo ? comp > S(0) : comp < S(0)) ? S(1) : S(-1);
-        const int step = xw ? (lo ? 1 : -1) : (lo ? LC : -LC);
-        const int64_t vin = (int64_t)(j + (xw ? 0 : (lo ? 1 : -1))) * (g.Nx + 1) + i + (xw ? (lo ? 1 : -1) : 0);
-        const int w0 = xw ? (lo ? o + 1 : o) : (lo ? o + LC : o), w1 = w0 + (xw ? LC : 1);
-        v = -sg * cv.te * (S(0.5) * (tu[w0] + tu[w1])) - node(o + step, cv.dv[vin]);
+        const bool x = wk <= 2, lo = wk == 1 || wk == 3;
+        const int o = wvy * LC + wvx, step = x ? (lo ? 1 : -1) : (lo ? LC : -LC);
+        const int w0 = x ? (lo ? o + 1 : o) : (lo ? o + LC : o), w1 = w0 + (x ? LC : 1);
+        const S comp = x ? kmu[k] : keta[k];
+        const S ht = (lo ? comp > S(0) : comp < S(0)) ? S(-0.5) * cv.te : S(0.5) * cv.te;
+        tv[wvy * LV + wvx] = fma(ht, tu[w0] + tu[w1], -node(o + step, wd));
       }
-      tv[e] = v;
     }
     group_sync<NT, G>(gq);
     if (live) {
-      const int o = ly * LV + lx;
-      const S v00 = tv[o], v10 = tv[o + 1], v01 = tv[o + LV], v11 = tv[o + LV + 1];
+      const S v10 = tv[ov + 1], v01 = tv[ov + LV], v11 = tv[ov + LV + 1];
+      if (edge) v00 = tv[ov];
       S div;
-      if (!wall) {
+      if (!edge) {
         div = fma(a, v11 - v00, bb * (v10 - v01));
       } else {
-        // (E_cell not from tu: the next pair's values may be on their way into it)
-        const CellSides<S> cs = cell_sides<S>(D, cv, k, pc, qc);
-        div = kmu[k] * cv.h2x * (cs.wL * (v00 + v01) + cs.wR * (v10 + v11)) +
-              keta[k] * cv.h2y * (cs.wB * (v00 + v10) + cs.wT * (v01 + v11)) + cs.ed() * (ec + rc);
+        div = fma(kmu[k], fma(cL, v00 + v01, cR * (v10 + v11)), keta[k] * fma(cB, v00 + v10, cT * (v01 + v11)));
+        const S ed = (wl || wr ? kex[k] : S(0)) + (wb || wt ? key[k] : S(0));
+        div = fma(ed, uc, div);
       }
-      const int64_t o2 = (int64_t)k * nc + c;
       S y = fma(kc, div, PRED ? fma(A, ec, arc) : A * ec);
       if (RES) y = bk - y;
       if (PRED) {
@@ -217,8 +246,8 @@ __global__ void __launch_bounds__(TX * TY * G) k2_op(D2 D, CV<S> cv, const S* __
           rows[k * NT + tid] = y;
         }
       }
-      if (!PREC) out[o2] = y;
-      else if (!PRED) out[o2] = ws * y * gik;
+      if (!PREC) out[k * nc + c] = y;
+      else if (!PRED) out[k * nc + c] = ws * y * gik;
     }
   }
   if (!PRED) return;
@@ -236,7 +265,7 @@ __global__ void __launch_bounds__(TX * TY * G) k2_op(D2 D, CV<S> cv, const S* __
     }
   }
   if (!live) return;
-  const int64_t orho = (int64_t)K * nc + c;
+  const int orho = K * nc + c;
   S rr = fma(al, rc, st);
   if (RES) rr = b[orho] - rr;
   if (!PREC) {
@@ -247,16 +276,15 @@ __global__ void __launch_bounds__(TX * TY * G) k2_op(D2 D, CV<S> cv, const S* __
   if (gq == 0) out[orho] = ws * rho;
 #pragma unroll 4
   for (int k = gq; k < K; k += G) {
-    const int64_t o2 = (int64_t)k * nc + c;
-    out[o2] = ws * fma(-(al + cv.gd[o2]), rho, rows[k * NT + tid]) * cv.gdi[o2];
+    const int o = k * nc + c;
+    out[o] = ws * fma(-(al + cv.gd[o]), rho, rows[k * NT + tid]) * cv.gdi[o];
   }
 }
 
 // ----------------------------------------------------------------------------- Gram-Schmidt
 // Streaming kernels over the basis: 16-byte loads (the vectors start on 16-byte boundaries,
 // a last partial group is done by single threads), one full wave of blocks.  Bound: HBM, or
-// the L2 where the basis fits; on small grids the fixed cost of the block sums, so the blocks
-// are as few as leave every thread a few groups of 16 bytes (vec_blocks).
+// the L2 where the basis fits; on small grids the latency of a turn and of the block sums.
 constexpr int kVecBlocks = 4 * 152;   // at most: block parts of a value
 
 template <typename S> struct Vec16;
@@ -474,59 +502,51 @@ __device__ __forceinline__ void krylov_column(KState* ks, int j, double hn2, KSt
 // again (binary64: when little of it is left, so that the rounding of the first pass weighs:
 // |w|^2 <= 1e-2 |w before|^2; binary32 cycles, which only have to gain 1e5 and whose restarts
 // are binary64, never); the last pass finishes the column.
-template <typename S>
-__global__ void __launch_bounds__(kThreads, 2) k2_axpy(S* __restrict__ w, const S* __restrict__ V, int64_t ld, int j,
-                                                       int64_t n, double* __restrict__ part, KState* ks,
-                                                       unsigned* count, int pass, KStop sp, KPin* pin) {
+// C: vectors of a chunk, loaded together (past the last one it is loaded again, with a zero
+// coefficient); U groups of 16 bytes per thread and turn.
+template <typename S, int C>
+__global__ void __launch_bounds__(kThreads, C <= 4 ? 4 : C <= 8 ? 3 : 2)
+    k2_axpy(S* __restrict__ w, const S* __restrict__ V, int64_t ld, int j, int64_t n, double* __restrict__ part,
+            KState* ks, unsigned* count, int pass, KStop sp, KPin* pin) {
   if (ks->stop || (pass == 2 && !ks->reorth)) return;
-  constexpr int N = Vec16<S>::N;
-  __shared__ S cf[kMaxRestart2 + 1];
+  constexpr int N = Vec16<S>::N, U = C <= 4 || (C <= 8 && sizeof(S) == 4) ? 2 : 1;
+  __shared__ S cf[kMaxRestart2 + 16];
   const int nv = j + 1;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) cf[i] = S(-ks->coef[i]);
+  for (int i = threadIdx.x; i < kMaxRestart2 + 16; i += blockDim.x) cf[i] = i < nv ? S(-ks->coef[i]) : S(0);
   __syncthreads();
   S nrm = S(0);
-  const int64_t ng = n / N;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ng; q += (int64_t)gridDim.x * blockDim.x) {
-    S a[N], a2[N];
-    load16(w + q * N, a);
+  const int64_t ng = n / N, nt = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ng; q += nt * U) {
+    S a[U][N];
 #pragma unroll
-    for (int e = 0; e < N; ++e) a2[e] = S(0);
-    const S* Vq = V + q * N;
-    int i = 0;
-    for (; i + 8 <= nv; i += 8) {
-      S v[8][N];
+    for (int u = 0; u < U; ++u) load16(w + min(q + u * nt, ng - 1) * N, a[u]);
+    for (int i0 = 0; i0 < nv; i0 += C) {
+      S v[U][C][N];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) load16(Vq + (int64_t)(i + t) * ld, v[t]);
+      for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int t = 0; t < 8; t += 2)
+        for (int t = 0; t < C; ++t)
+          load16(V + (int64_t)min(i0 + t, nv - 1) * ld + min(q + u * nt, ng - 1) * N, v[u][t]);
 #pragma unroll
-        for (int e = 0; e < N; ++e) {
-          a[e] = fma(cf[i + t], v[t][e], a[e]);
-          a2[e] = fma(cf[i + t + 1], v[t + 1][e], a2[e]);
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < N; ++e) {   // two sums per element: shorter chains
+          S s0 = S(0), s1 = S(0);
+#pragma unroll
+          for (int t = 0; t < C; t += 2) {
+            s0 = fma(cf[i0 + t], v[u][t][e], s0);
+            s1 = fma(cf[i0 + t + 1], v[u][t + 1][e], s1);
+          }
+          a[u][e] += s0 + s1;
         }
     }
-    for (; i + 2 <= nv; i += 2) {
-      S v[2][N];
-      load16(Vq + (int64_t)i * ld, v[0]);
-      load16(Vq + (int64_t)(i + 1) * ld, v[1]);
 #pragma unroll
-      for (int e = 0; e < N; ++e) {
-        a[e] = fma(cf[i], v[0][e], a[e]);
-        a2[e] = fma(cf[i + 1], v[1][e], a2[e]);
-      }
-    }
-    if (i < nv) {
-      S v[N];
-      load16(Vq + (int64_t)i * ld, v);
+    for (int u = 0; u < U; ++u) {
+      if (q + u * nt >= ng) continue;
 #pragma unroll
-      for (int e = 0; e < N; ++e) a[e] = fma(cf[i], v[e], a[e]);
+      for (int e = 0; e < N; ++e) nrm = fma(a[u][e], a[u][e], nrm);
+      *reinterpret_cast<typename Vec16<S>::T*>(w + (q + u * nt) * N) = *reinterpret_cast<typename Vec16<S>::T*>(a[u]);
     }
-#pragma unroll
-    for (int e = 0; e < N; ++e) {
-      a[e] += a2[e];
-      nrm = fma(a[e], a[e], nrm);
-    }
-    *reinterpret_cast<typename Vec16<S>::T*>(w + q * N) = *reinterpret_cast<typename Vec16<S>::T*>(a);
   }
   if (blockIdx.x == 0 && (int64_t)threadIdx.x < n - ng * N) {
     const int64_t e = ng * N + threadIdx.x;
