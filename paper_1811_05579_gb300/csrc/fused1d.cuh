@@ -61,10 +61,11 @@ struct FSmem {
   float endr[2][2][32];                                 // published: r'_F, r'_L
   float coup[2][2][32];                                 // published: a at the first cell, c at the last
   float xlr[2][32];                                     // e at c0 - 1 and at c0 + kFS, per angle
-  float vk[32], v2k[32], wvk[32], wvkl[32];            // per-angle constants (0 past M); wvkl:
+  float vk[32], v2k[32], wvk[32], wvkl[32], nwv2[32];  // per-angle constants (0 past M); nwv2: -wvk vk; wvkl:
                                                         // w v - wvk (binary32 low part)
   double vkd[32], wvkd[32];
   double wib[2][32], wgn[2][32], won[2][32], wdl[2];   // inflow wall rows (f_load_cells)
+  double wkv[2][32], wbv[2][32], wdat[2][32], wcf[2][5];   // and their right-hand sides (f_wall_rhs)
   double fl[kFS];                                       // flux sums of the last pass
   double fdat[kFS];                                     // data part of the flux (data passes)
   // the correction's flux (sigma_0/T^3): node coefficients d* of V* = (U*)^{3/4} at the
@@ -86,7 +87,7 @@ struct FSmem {
   double xmx[2];                                        // the slice's max |x|, per restart parity
   double xmall;                                         // the cluster's max |x|
   double wall[2][32];                                   // wall-row right-hand sides (double)
-  double red[kFW][kMaxRestart + 2];                     // per-warp partial sums
+  double red[4][kMaxRestart + 2];                       // per-warp partial sums (kGW warps)
   double part[2][kMaxRestart + 2];                      // cluster partials (double-buffered)
   double sums[kMaxRestart + 2];
   // binary64 preconditioner: reduced rows of the 32 lane chunks (64 rows), interface
@@ -110,9 +111,17 @@ static_assert(2 * sizeof(FSmem::ra) >= (kFS + 2) * sizeof(double), "room for V*"
 // Per-CTA geometry.
 struct FGeo {
   int ii, q, Q;         // instance, slice, slices in the cluster
+  int nl;               // cells of the slice inside the grid (<= 0: none)
   int64_t c0, co;       // first cell of the slice (instance-local), instance cell offset
   int N, M;
 };
+
+// Barrier over the instance's CTAs: the cluster's, or for a single CTA the block's (a cluster
+// barrier of one CTA costs ~500 cycles more, five times per Krylov step).
+__device__ __forceinline__ void f_sync(cg::cluster_group& cl) {
+  if (cl.num_blocks() > 1) cl.sync();
+  else __syncthreads();
+}
 
 // Cluster reductions.  The binary64 pipe is the scarce resource (one warp instruction
 // holds a sub-partition's pipe for many cycles), so the slice part runs on warps 0..3, one
@@ -148,15 +157,32 @@ __device__ __forceinline__ double f_warp_rs(double (&a)[S], int lane, int& vi) {
 
 // Warp part of the slice sums for S slots (ns <= S live): writes sm.red[wid][0..ns-1].
 template <int S, class FS>
-__device__ __forceinline__ void f_slice_rs(FSmem& sm, int ns, FS sterm) {
+__device__ __forceinline__ void f_slice_rs(FSmem& sm, int ns, int nl, FS sterm) {
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   double a[S];
+  static_assert(kGC == 4, "four groups of cells");
+  if (nl > (kGC - 1) * 32 * kGW) {
 #pragma unroll
-  for (int i = 0; i < S; ++i) {
-    a[i] = 0.0;
-    if (i < ns) {
+    for (int i = 0; i < S; ++i) {
+      a[i] = 0.0;
+      if (i < ns) {
 #pragma unroll
-      for (int c = 0; c < kGC; ++c) a[i] += sterm(i, t + c * 32 * kGW);
+        for (int c = 0; c < kGC; ++c) a[i] += sterm(i, t + c * 32 * kGW);
+      }
+    }
+  } else {   // (the terms past the grid are 0: the groups of cells inside it only)
+    const bool g1 = nl > 32 * kGW, g2 = nl > 2 * 32 * kGW;
+#pragma unroll
+    for (int i = 0; i < S; ++i) a[i] = i < ns ? 0.0 + sterm(i, t) : 0.0;
+    if (g1) {
+#pragma unroll
+      for (int i = 0; i < S; ++i)
+        if (i < ns) a[i] += sterm(i, t + 32 * kGW);
+    }
+    if (g2) {
+#pragma unroll
+      for (int i = 0; i < S; ++i)
+        if (i < ns) a[i] += sterm(i, t + 2 * 32 * kGW);
     }
   }
   int vi;
@@ -165,19 +191,20 @@ __device__ __forceinline__ void f_slice_rs(FSmem& sm, int ns, FS sterm) {
   if ((lane & lowbits) == 0 && vi < ns) sm.red[wid][vi] = r;
 }
 
+// (nl: the slice's cells inside the grid; the terms are 0 past them.)
 // ns <= NS sums of sterm(i, c) (i < ns) and, if MX, the maximum of mterm(c) >= 0 over the
 // cluster's cells (c the slice cell); results in sm.sums[0..ns-1] and sm.sums[ns] for every
 // thread.  Every thread takes part; par selects the half of the double buffer.
 template <int NS, bool MX, class FS, class FM>
-__device__ void f_reduce(FSmem& sm, cg::cluster_group& cl, int& par, int ns, FS sterm, FM mterm) {
+__device__ void f_reduce(FSmem& sm, cg::cluster_group& cl, int nl, int& par, int ns, FS sterm, FM mterm) {
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   if (wid < kGW) {
     if (NS > 0 && ns > 0) {
-      if (NS <= 1 || ns <= 1) f_slice_rs<1>(sm, ns, sterm);
-      else if (NS <= 2 || ns <= 2) f_slice_rs<(NS < 2 ? 1 : 2)>(sm, ns, sterm);
-      else if (NS <= 4 || ns <= 4) f_slice_rs<(NS < 4 ? 1 : 4)>(sm, ns, sterm);
-      else if (NS <= 8 || ns <= 8) f_slice_rs<(NS < 8 ? 1 : 8)>(sm, ns, sterm);
-      else f_slice_rs<(NS < 16 ? 1 : 16)>(sm, ns, sterm);
+      if (NS <= 1 || ns <= 1) f_slice_rs<1>(sm, ns, nl, sterm);
+      else if (NS <= 2 || ns <= 2) f_slice_rs<(NS < 2 ? 1 : 2)>(sm, ns, nl, sterm);
+      else if (NS <= 4 || ns <= 4) f_slice_rs<(NS < 4 ? 1 : 4)>(sm, ns, nl, sterm);
+      else if (NS <= 8 || ns <= 8) f_slice_rs<(NS < 8 ? 1 : 8)>(sm, ns, nl, sterm);
+      else f_slice_rs<(NS < 16 ? 1 : 16)>(sm, ns, nl, sterm);
     }
     if (MX) {
       long long m = 0;
@@ -200,7 +227,12 @@ __device__ void f_reduce(FSmem& sm, cg::cluster_group& cl, int& par, int ns, FS 
     } else {
       v = (sm.red[0][t] + sm.red[1][t]) + (sm.red[2][t] + sm.red[3][t]);
     }
-    sm.part[par][t] = v;
+    if (cl.num_blocks() == 1) sm.sums[t] = v;
+    else sm.part[par][t] = v;
+  }
+  if (cl.num_blocks() == 1) {   // (uniform)
+    __syncthreads();
+    return;
   }
   cl.sync();
   // 16 lanes per value, lane r reading rank r's partial
@@ -249,14 +281,13 @@ __device__ __forceinline__ void f_coef(const FSmem& sm, int jl, float v, float v
 // w + kFW with lane = row; the rows are kept scaled to a unit diagonal, so a level takes the
 // neighbours' (a, c, r) by shuffles and one reciprocal.  The arrays are padded to 33
 // columns, so that a warp's column reads hit 32 banks.  Every thread takes part.
-template <int NR>
-__device__ __forceinline__ void f_pcr(FSmem& sm, int n) {
-  static_assert(2 * kFW == 32, "two angles per warp");
+template <int NR, int H>
+__device__ __forceinline__ void f_pcr_angles(FSmem& sm, int n) {
   const int i = threadIdx.x & 31, w = threadIdx.x >> 5;
   const bool live = i < n;
-  float a[2], c[2], r[2][NR];
+  float a[H], c[H], r[H][NR];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < H; ++h) {
     const int k = w + h * kFW;
     if (live) {
       const float ib = __frcp_rn(sm.rb[i][k]);
@@ -274,7 +305,7 @@ __device__ __forceinline__ void f_pcr(FSmem& sm, int n) {
   for (int st = 1; st < n; st <<= 1) {
     const bool hl = i >= st, hr = i + st < n;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < H; ++h) {
       float al = __shfl_up_sync(0xffffffffu, a[h], st), cl = __shfl_up_sync(0xffffffffu, c[h], st);
       float ar = __shfl_down_sync(0xffffffffu, a[h], st), cr = __shfl_down_sync(0xffffffffu, c[h], st);
       float rl[NR], rr[NR];
@@ -295,13 +326,21 @@ __device__ __forceinline__ void f_pcr(FSmem& sm, int n) {
   }
   if (live) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < H; ++h) {
       const int k = w + h * kFW;
       sm.rr[i][k] = r[h][0];
       if (NR > 1) sm.rg[i][k] = r[h][1];
       if (NR > 2) sm.rh[i][k] = r[h][2];
     }
   }
+}
+// The angles past M (right-hand sides 0) are left as they are.
+template <int NR>
+__device__ __forceinline__ void f_pcr(FSmem& sm, int n, int M) {
+  static_assert(2 * kFW == 32, "two angles per warp");
+  const int w = threadIdx.x >> 5;
+  if (w + kFW < M) f_pcr_angles<NR, 2>(sm, n);
+  else if (w < M) f_pcr_angles<NR, 1>(sm, n);
   __syncthreads();
 }
 
@@ -312,51 +351,56 @@ __device__ void f_line_solve(FSmem& sm, cg::cluster_group& cl, const FGeo& G, in
   const int k = threadIdx.x & 31, w = threadIdx.x >> 5;
   const float v = sm.vk[k], v2 = sm.v2k[k];
   const int row0 = w * kFL;
+  // A chunk past the grid (identity rows, right-hand side 0) has nothing to eliminate: its warp
+  // leaves the issue slots to the others.
+  const bool dead = row0 >= G.nl;
   // (1) backward elimination of the chunk's interior from its last cell:
   //     x_u = rt_u - at_u x_{u-1} - ct_u x_e, down to u = 1 (the S row's partner)
   float rt = 0.0f, at = 0.0f, ct = 0.0f;
-#pragma unroll
-  for (int u = kFL - 2; u >= 1; --u) {
-    float a, b, c;
-    f_coef(sm, row0 + u + 1, v, v2, a, b, c);
-    const float r = sm.x[row0 + u][k];
-    float den, num, ctv;
-    if (u == kFL - 2) {
-      den = b;
-      num = r;
-      ctv = c;
-    } else {
-      den = fmaf(-c, at, b);
-      num = fmaf(-c, rt, r);
-      ctv = -c * ct;
-    }
-    const float inv = f_rcp(den);
-    rt = num * inv;
-    at = a * inv;
-    ct = ctv * inv;
-  }
   // (2) forward elimination: x_u = rh_u - ch_u x_{u+1} - ah_u x_s (rh_u kept in sm.x)
   float rhp = 0.0f, chp = 0.0f, ahp = 0.0f;
+  if (!dead) {
 #pragma unroll
-  for (int u = 1; u <= kFL - 2; ++u) {
-    float a, b, c;
-    f_coef(sm, row0 + u + 1, v, v2, a, b, c);
-    const float r = sm.x[row0 + u][k];
-    float den, ahv, num;
-    if (u == 1) {
-      den = b;
-      ahv = a;
-      num = r;
-    } else {
-      den = fmaf(-a, chp, b);
-      ahv = -a * ahp;
-      num = fmaf(-a, rhp, r);
+    for (int u = kFL - 2; u >= 1; --u) {
+      float a, b, c;
+      f_coef(sm, row0 + u + 1, v, v2, a, b, c);
+      const float r = sm.x[row0 + u][k];
+      float den, num, ctv;
+      if (u == kFL - 2) {
+        den = b;
+        num = r;
+        ctv = c;
+      } else {
+        den = fmaf(-c, at, b);
+        num = fmaf(-c, rt, r);
+        ctv = -c * ct;
+      }
+      const float inv = f_rcp(den);
+      rt = num * inv;
+      at = a * inv;
+      ct = ctv * inv;
     }
-    const float inv = f_rcp(den);
-    chp = c * inv;
-    ahp = ahv * inv;
-    rhp = num * inv;
-    sm.x[row0 + u][k] = rhp;
+#pragma unroll
+    for (int u = 1; u <= kFL - 2; ++u) {
+      float a, b, c;
+      f_coef(sm, row0 + u + 1, v, v2, a, b, c);
+      const float r = sm.x[row0 + u][k];
+      float den, ahv, num;
+      if (u == 1) {
+        den = b;
+        ahv = a;
+        num = r;
+      } else {
+        den = fmaf(-a, chp, b);
+        ahv = -a * ahp;
+        num = fmaf(-a, rhp, r);
+      }
+      const float inv = f_rcp(den);
+      chp = c * inv;
+      ahp = ahv * inv;
+      rhp = num * inv;
+      sm.x[row0 + u][k] = rhp;
+    }
   }
   {
     float as, bs, cs, ae, be, ce;
@@ -381,7 +425,7 @@ __device__ void f_line_solve(FSmem& sm, cg::cluster_group& cl, const FGeo& G, in
     if (w == kFW - 1) sm.coup[par][1][k] = ce;         // c at its last cell
   }
   __syncthreads();
-  f_pcr<3>(sm, kFR);
+  f_pcr<3>(sm, kFR, G.M);
   // the slice's 2x2 Schur complement on (first, last): S = Z^{-1}, Z = [[g0, h0], [g1, h1]]
   if (w == 0) {
     const float z00 = sm.rg[0][k], z0n = sm.rh[0][k], zn0 = sm.rg[kFR - 1][k], znn = sm.rh[kFR - 1][k];
@@ -396,7 +440,7 @@ __device__ void f_line_solve(FSmem& sm, cg::cluster_group& cl, const FGeo& G, in
     sm.endr[par][0][k] = S11 * y0 + S12 * y1;
     sm.endr[par][1][k] = S21 * y0 + S22 * y1;
   }
-  cl.sync();
+  f_sync(cl);
   // interface system of all slices, rows [F_0, L_0, F_1, L_1, ...] per angle:
   //   a_q L_{q-1} + S11 F_q + S12 L_q = r'_F,   S21 F_q + S22 L_q + c_q F_{q+1} = r'_L
   // (built in every CTA from the gathered values into ra..rr; the slice's own y, g, h
@@ -455,7 +499,7 @@ __device__ void f_line_solve(FSmem& sm, cg::cluster_group& cl, const FGeo& G, in
   __syncthreads();
   // this CTA's couplings (read before the interface solve reuses the arrays)
   const float a_first = sm.coup[par][0][k], c_last = sm.coup[par][1][k];
-  f_pcr<1>(sm, n2);
+  f_pcr<1>(sm, n2, G.M);
   const float Lp = (G.q > 0) ? sm.rr[2 * G.q - 1][k] : 0.0f;
   const float Fn = (G.q < Q - 1) ? sm.rr[2 * G.q + 2][k] : 0.0f;
   __syncthreads();
@@ -477,9 +521,9 @@ __device__ void f_line_solve(FSmem& sm, cg::cluster_group& cl, const FGeo& G, in
   __syncthreads();
   // back substitution of the chunk: the forward factors ch, ah (matrix only) recomputed
   // into registers, then x_u = rh_u - ch_u x_{u+1} - ah_u x_s from the last cell down
-  const float xs = sm.rr[2 * w][k], xe = sm.rr[2 * w + 1][k];
-  float ch[kFL - 2], ah[kFL - 2];
-  {
+  if (!dead) {
+    const float xs = sm.rr[2 * w][k], xe = sm.rr[2 * w + 1][k];
+    float ch[kFL - 2], ah[kFL - 2];
     float chv = 0.0f, ahv = 0.0f;
 #pragma unroll
     for (int u = 1; u <= kFL - 2; ++u) {
@@ -492,14 +536,14 @@ __device__ void f_line_solve(FSmem& sm, cg::cluster_group& cl, const FGeo& G, in
       ch[u - 1] = chv;
       ah[u - 1] = ahv;
     }
-  }
-  sm.x[row0][k] = xs;
-  sm.x[row0 + kFL - 1][k] = xe;
-  float xn = xe;
+    sm.x[row0][k] = xs;
+    sm.x[row0 + kFL - 1][k] = xe;
+    float xn = xe;
 #pragma unroll
-  for (int u = kFL - 2; u >= 1; --u) {
-    xn = fmaf(-ch[u - 1], xn, fmaf(-ah[u - 1], xs, sm.x[row0 + u][k]));
-    sm.x[row0 + u][k] = xn;
+    for (int u = kFL - 2; u >= 1; --u) {
+      xn = fmaf(-ch[u - 1], xn, fmaf(-ah[u - 1], xs, sm.x[row0 + u][k]));
+      sm.x[row0 + u][k] = xn;
+    }
   }
   __syncthreads();
 }
@@ -524,6 +568,7 @@ __device__ void f_load_cells(FSmem& sm, const Dev& D, const Inst& I, const FGeo&
     sm.v2k[k] = (float)(v * v);
     sm.wvk[k] = (float)(w * v);
     sm.wvkl[k] = (float)(w * v - (double)(float)(w * v));
+    sm.nwv2[k] = -sm.wvk[k] * sm.vk[k];
     sm.vkd[k] = v;
     sm.wvkd[k] = w * v;
     // inflow wall rows of this slice (per angle, fixed for the solve): 1/b of the wall
@@ -539,7 +584,20 @@ __device__ void f_load_cells(FSmem& sm, const Dev& D, const Inst& I, const FGeo&
         sm.wgn[side][k] = ka ? v2 * (side == 0 ? D.cf.gu[g] : D.cf.gl[g]) / bw : 0.0;
         const float* Ok = (const float*)D.O + I.nelem_off + (int64_t)k * (G.N + 1);
         sm.won[side][k] = ka ? (double)(D.fc.od[G.co + ni] * Ok[ni]) : 0.0;
-        if (k == 0) sm.wdl[side] = D.cf.dlx[G.co + ni];
+        // right-hand side (f_wall_rhs): kappa v (2/eps)/dx, the inflow intensity, the data term
+        const float* Ek = (const float*)D.Eh + I.elem_off + (int64_t)k * G.N;
+        const double on = sm.won[side][k], o = side == 0 ? 2.0 * on : -2.0 * on;
+        sm.wkv[side][k] = ka ? D.cf.kdx[g] * v * I.two_eps : 0.0;
+        sm.wbv[side][k] = ka ? (side == 0 ? D.bL[I.ang_off + k] : D.bR[I.ang_off + k]) : 0.0;
+        sm.wdat[side][k] = ka ? D.cf.kcd[g] * (double)Ek[jw] - D.cf.kdx[g] * v * o : 0.0;
+        if (k == 0) {
+          sm.wdl[side] = D.cf.dlx[G.co + ni];
+          sm.wcf[side][0] = D.cf.alpha[g];
+          sm.wcf[side][1] = D.cf.gl[g];
+          sm.wcf[side][2] = D.cf.gu[g];
+          sm.wcf[side][3] = D.cf.sac[g] + D.cf.kcd[g] * I.a * I.c;
+          sm.wcf[side][4] = D.U[g];
+        }
       }
     }
   }
@@ -686,6 +744,7 @@ __device__ void f_stage_data(FSmem& sm, const Dev& D, const Inst& I, const FGeo&
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float* fd = D.fdata + I.fd_off + (G.c0 + w * kFL) * 32;
   if (!stage) {
+    if (w * kFL >= G.nl) return;   // (zeros, still in place)
 #pragma unroll 8
     for (int u = 0; u < kFL; ++u) sm.x[w * kFL + u][lane] = fd[u * 32 + lane];
     __syncwarp();
@@ -739,26 +798,21 @@ __device__ void f_stage_data(FSmem& sm, const Dev& D, const Inst& I, const FGeo&
 
 // Right-hand side of the inflow wall row j (0 or N-1) for angle k in binary64:
 //   P1 - v^2 P2 + kappa v (2/eps)(b - x)/dx  [+ kappa/(c dt) Eh^n - kappa v o/dx on data passes,
-//   o = 2 o_1 (left) or -2 o_{N-1} (right)] (the O(eps) difference is formed in double).
+//   o = 2 o_1 (left) or -2 o_{N-1} (right)] (the O(eps) difference is formed in double);
+// everything but x from the solve's constants in shared memory (f_load_cells).
 template <bool FULL>
-__device__ double f_wall_rhs(const Dev& D, const Inst& I, const FGeo& G, const FVec& X, int64_t j, int k) {
-  const int64_t N = G.N, g = G.co + j;
-  const double v = D.v[I.ang_off + k], v2 = v * v;
+__device__ double f_wall_rhs(const FSmem& sm, const FGeo& G, const FVec& X, int side, int k) {
+  const int64_t N = G.N, j = side == 0 ? 0 : N - 1;
   const double xj = f_x<FULL>(X, G, j), xl = j > 0 ? f_x<FULL>(X, G, j - 1) : 0.0,
                xr = j < N - 1 ? f_x<FULL>(X, G, j + 1) : 0.0;
-  double p1 = -D.cf.alpha[g] * xj;
-  if (FULL) p1 += (D.cf.sac[g] + D.cf.kcd[g] * I.a * I.c) * D.U[g];
-  const double p2 = D.cf.gl[g] * (xj - xl) + D.cf.gu[g] * (xj - xr);
-  const double b = FULL ? ((j == 0) ? D.bL[I.ang_off + k] : D.bR[I.ang_off + k]) : 0.0;
-  double r = p1 - v2 * p2 + D.cf.kdx[g] * v * I.two_eps * (b - xj);
-  if (FULL) {
-    const float* Ok = (const float*)D.O + I.nelem_off + (int64_t)k * (N + 1);
-    const float* Ek = (const float*)D.Eh + I.elem_off + (int64_t)k * N;
-    const int64_t ni = (j == 0) ? 1 : N - 1;
-    const double on = (double)(D.fc.od[G.co + ni] * Ok[ni]);
-    const double o = (j == 0) ? 2.0 * on : -2.0 * on;
-    r += D.cf.kcd[g] * (double)Ek[j] - D.cf.kdx[g] * v * o;
-  }
+  const double* c = sm.wcf[side];
+  const double v = sm.vkd[k];
+  double p1 = -c[0] * xj;
+  if (FULL) p1 += c[3] * c[4];
+  const double p2 = c[1] * (xj - xl) + c[2] * (xj - xr);
+  const double b = FULL ? sm.wbv[side][k] : 0.0;
+  double r = p1 - v * v * p2 + sm.wkv[side][k] * (b - xj);
+  if (FULL) r += sm.wdat[side][k];
   return r;
 }
 
@@ -769,7 +823,7 @@ __device__ double f_wall_rhs(const Dev& D, const Inst& I, const FGeo& G, const F
 template <bool FULL>
 __device__ void f_pass(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Inst& I, const FGeo& G,
                        const double* xg, int& par, bool stage = false) {
-  cl.sync();   // xg complete on every slice (halo reads)
+  f_sync(cl);   // xg complete on every slice (halo reads)
   FVec X{xg, 0.0, 0.0};
   if (!FULL) {
     // the direction's values next to the slice, from the neighbouring CTAs' shared memory
@@ -783,13 +837,16 @@ __device__ void f_pass(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Ins
   __syncthreads();
   const bool inflow = I.bc == GRTE_BC_INFLOW;
   const float v = sm.vk[k], v2 = sm.v2k[k];
-  // right-hand sides r = P1 - v^2 P2 - v P3 (+ data) of the chunk
-#pragma unroll 4
-  for (int u = 0; u < kFL; ++u) {
-    const int t = w * kFL + u;
-    float r = fmaf(-v, sm.P3[t], fmaf(-v2, sm.P2[t], sm.P1[t]));
-    if (FULL) r += sm.x[t][k];
-    sm.x[t][k] = (k < G.M) ? r : 0.0f;
+  // right-hand sides r = P1 - v^2 P2 - v P3 (+ data) of the chunk (a chunk past the grid keeps the
+  // zeros of the first data pass)
+  if (w * kFL < G.nl || (FULL && stage)) {
+#pragma unroll 8
+    for (int u = 0; u < kFL; ++u) {
+      const int t = w * kFL + u;
+      float r = fmaf(-v, sm.P3[t], fmaf(-v2, sm.P2[t], sm.P1[t]));
+      if (FULL) r += sm.x[t][k];
+      sm.x[t][k] = (k < G.M) ? r : 0.0f;
+    }
   }
   // inflow wall rows in double
   if (inflow && k < G.M) {
@@ -797,7 +854,7 @@ __device__ void f_pass(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Ins
       const int64_t jw = side == 0 ? 0 : N - 1;
       const int64_t tl = jw - G.c0;
       if (tl >= 0 && tl < kFS && (int)(tl / kFL) == w) {
-        const double r = f_wall_rhs<FULL>(D, I, G, X, jw, k);
+        const double r = f_wall_rhs<FULL>(sm, G, X, side, k);
         sm.wall[side][k] = r;
         sm.x[tl][k] = (float)r;
       }
@@ -848,10 +905,10 @@ __device__ void f_pass(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Ins
         // compensated binary32 sum (Knuth's two-sum): the rounding error of every addition
         // is carried in lo, so hi + lo holds the sum to about 2^-48 relative
         float hi = 0.0f, lo = 0.0f;
+#pragma unroll 8
         for (int kk = 0; kk < G.M; ++kk) {
           const float ej = sm.x[t][kk];
-          const float wv2k = -sm.wvk[kk] * sm.vk[kk];
-          const float a = wv2k * (dR * (xr[kk] - ej) - dL * (ej - xl[kk]));
+          const float a = sm.nwv2[kk] * (dR * (xr[kk] - ej) - dL * (ej - xl[kk]));
           const float sN = hi + a;
           const float bb = sN - hi;
           lo += (hi - (sN - bb)) + (a - bb);
@@ -860,9 +917,10 @@ __device__ void f_pass(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Ins
         sm.fl[t] += sm.fdat[t] + ((double)hi + (double)lo);
       } else {
         float acc = (float)sm.fl[t];
+#pragma unroll 8
         for (int kk = 0; kk < G.M; ++kk) {
           const float ej = sm.x[t][kk];
-          acc += -sm.wvk[kk] * sm.vk[kk] * (dR * (xr[kk] - ej) - dL * (ej - xl[kk]));
+          acc += sm.nwv2[kk] * (dR * (xr[kk] - ej) - dL * (ej - xl[kk]));
         }
         sm.fl[t] = (double)acc;
       }
@@ -871,12 +929,37 @@ __device__ void f_pass(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Ins
   __syncthreads();
 }
 
-// Right-hand side of row il (and row ir) of a 64-row system held two rows per lane of
-// warp 0 (rows 2 lane, 2 lane + 1 in v0, v1).
-__device__ __forceinline__ double f_row(double v0, double v1, int i) {
-  const int src = (i < 0 ? 0 : (i > 63 ? 63 : i));
-  const double a = __shfl_sync(0xffffffffu, v0, src >> 1), b = __shfl_sync(0xffffffffu, v1, src >> 1);
-  return (src & 1) ? b : a;
+// Rows i - st and i + st of a 64-row system held two rows per lane of a warp (rows 2 lane + p in
+// v[p]); st a power of two: the neighbours of a row are in the other slot for st = 1 and in the
+// same slot, st/2 lanes away, above.  (Past the ends: any value; the caller masks.)
+__device__ __forceinline__ double f_row_l(const double (&v)[2], int p, int st) {
+  if (st == 1) return p ? v[0] : __shfl_up_sync(0xffffffffu, v[1], 1);
+  return __shfl_up_sync(0xffffffffu, v[p], st >> 1);
+}
+__device__ __forceinline__ double f_row_r(const double (&v)[2], int p, int st) {
+  if (st == 1) return p ? __shfl_down_sync(0xffffffffu, v[0], 1) : v[1];
+  return __shfl_down_sync(0xffffffffu, v[p], st >> 1);
+}
+
+// One right-hand side of the reduced 64-row system (two rows per lane of one warp) with the
+// stored PCR multipliers and diagonal reciprocals; in place.
+__device__ __forceinline__ void f_pcr64(const FSmem& sm, double (&r)[2], int lane) {
+#pragma unroll
+  for (int l = 0; l < 6; ++l) {
+    const int st = 1 << l;
+    double n[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int i = 2 * lane + p;
+      // (pk1, pk2 are 0 where the neighbour does not exist)
+      const double L = f_row_l(r, p, st), R = f_row_r(r, p, st);
+      n[p] = r[p] - sm.pk1[l][i] * L - sm.pk2[l][i] * R;
+    }
+    r[0] = n[0];
+    r[1] = n[1];
+  }
+  r[0] *= sm.pib[2 * lane];
+  r[1] *= sm.pib[2 * lane + 1];
 }
 
 // Cell slot (within a lane's 16-cell chunk) of row i of the preconditioner's level-B
@@ -980,59 +1063,89 @@ __device__ void f_prec_factor(FSmem& sm, cg::cluster_group& cl, const Dev& D, co
     const double as = a[0], bs = b[0], cs = c[0], ae = a[7], be = b[7], ce = c[7];
     sm.pcs[lane] = cs;
     sm.pae[lane] = ae;
-    double ra0 = (lane == 0) ? 0.0 : as, rb0 = bs - cs * ac, rc0 = -cs * cc;
-    double ra1 = -ae * ahv[6], rb1 = be - ae * chv[6];
-    double rc1 = (lane == 31) ? 0.0 : ce;
-    double g0 = (lane == 0) ? 1.0 : 0.0, g1 = 0.0, h0 = 0.0, h1 = (lane == 31) ? 1.0 : 0.0;
-    const double af = __shfl_sync(0xffffffffu, as, 0), cl_ = __shfl_sync(0xffffffffu, ce, 31);
-    for (int l = 0, st = 1; st < 64; ++l, st <<= 1) {
-      double na[2], nb[2], nc[2], ng[2], nh[2];
+    // the chunk-end rows 2 lane, 2 lane + 1 of the reduced system, by (a, b, c)
+    double* const rr = lb;   // [3][64] (level B has read its rows into registers)
+    __syncwarp();
+    rr[2 * lane] = (lane == 0) ? 0.0 : as;
+    rr[2 * lane + 1] = -ae * ahv[6];
+    rr[64 + 2 * lane] = bs - cs * ac;
+    rr[64 + 2 * lane + 1] = be - ae * chv[6];
+    rr[128 + 2 * lane] = -cs * cc;
+    rr[128 + 2 * lane + 1] = (lane == 31) ? 0.0 : ce;
+    if (lane == 0) sm.paf = as;
+    if (lane == 31) sm.pcl = ce;
+  }
+  __syncthreads();
+  // PCR of the 64 rows on two warps (two sub-partitions' binary64 pipes): warp p has the rows
+  // 2 lane + p; the first level's neighbours are the other warp's rows, read from shared memory,
+  // all later levels' its own, st/2 lanes away
+  if (w < 2) {
+    const double* const rr = lb;
+    const int i = 2 * lane + w;
+    double a = rr[i], b = rr[64 + i], c = rr[128 + i];
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+      const int st = 1 << l;
+      const bool hl = i >= st, hr = i + st < 64;
+      double La, Lb, Lc, Ra, Rb, Rc;
+      if (l == 0) {
+        const int il = hl ? i - 1 : 0, ir = hr ? i + 1 : 63;
+        La = rr[il], Lb = rr[64 + il], Lc = rr[128 + il];
+        Ra = rr[ir], Rb = rr[64 + ir], Rc = rr[128 + ir];
+      } else {
+        La = __shfl_up_sync(0xffffffffu, a, st >> 1);
+        Lb = __shfl_up_sync(0xffffffffu, b, st >> 1);
+        Lc = __shfl_up_sync(0xffffffffu, c, st >> 1);
+        Ra = __shfl_down_sync(0xffffffffu, a, st >> 1);
+        Rb = __shfl_down_sync(0xffffffffu, b, st >> 1);
+        Rc = __shfl_down_sync(0xffffffffu, c, st >> 1);
+      }
+      const double k1 = hl ? a / Lb : 0.0, k2 = hr ? c / Rb : 0.0;
+      sm.pk1[l][i] = k1;
+      sm.pk2[l][i] = k2;
+      a = hl ? -La * k1 : 0.0;
+      c = hr ? -Rc * k2 : 0.0;
+      b = b - (hl ? Lc * k1 : 0.0) - (hr ? Ra * k2 : 0.0);
+    }
+    sm.pib[i] = 1.0 / b;
+  }
+  __syncthreads();
+  // the two unit spikes, each a right-hand side of its own, on two other sub-partitions
+  if (w == 1 || w == 2) {
+    double r[2] = {w == 1 && lane == 0 ? 1.0 : 0.0, w == 2 && lane == 31 ? 1.0 : 0.0};
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+      const int st = 1 << l;
+      double n[2];
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        const int i = 2 * lane + p, il = i - st, ir = i + st;
-        const bool hl = il >= 0, hr = ir < 64;
-        const double Lb = f_row(rb0, rb1, il), La = f_row(ra0, ra1, il), Lc = f_row(rc0, rc1, il);
-        const double Lg = f_row(g0, g1, il), Lh = f_row(h0, h1, il);
-        const double Rb = f_row(rb0, rb1, ir), Ra = f_row(ra0, ra1, ir), Rc = f_row(rc0, rc1, ir);
-        const double Rg = f_row(g0, g1, ir), Rh = f_row(h0, h1, ir);
-        const double a = p ? ra1 : ra0, b = p ? rb1 : rb0, c = p ? rc1 : rc0;
-        const double k1 = hl ? a / Lb : 0.0, k2 = hr ? c / Rb : 0.0;
-        sm.pk1[l][i] = k1;
-        sm.pk2[l][i] = k2;
-        na[p] = hl ? -La * k1 : 0.0;
-        nc[p] = hr ? -Rc * k2 : 0.0;
-        nb[p] = b - (hl ? Lc * k1 : 0.0) - (hr ? Ra * k2 : 0.0);
-        ng[p] = (p ? g1 : g0) - (hl ? Lg * k1 : 0.0) - (hr ? Rg * k2 : 0.0);
-        nh[p] = (p ? h1 : h0) - (hl ? Lh * k1 : 0.0) - (hr ? Rh * k2 : 0.0);
+        const int i = 2 * lane + p;
+        const double L = f_row_l(r, p, st), R = f_row_r(r, p, st);
+        n[p] = r[p] - (i >= st ? L * sm.pk1[l][i] : 0.0) - (i + st < 64 ? R * sm.pk2[l][i] : 0.0);
       }
-      ra0 = na[0]; ra1 = na[1]; rb0 = nb[0]; rb1 = nb[1]; rc0 = nc[0]; rc1 = nc[1];
-      g0 = ng[0]; g1 = ng[1]; h0 = nh[0]; h1 = nh[1];
+      r[0] = n[0];
+      r[1] = n[1];
     }
-    const double i0 = 1.0 / rb0, i1 = 1.0 / rb1;
-    sm.pib[2 * lane] = i0;
-    sm.pib[2 * lane + 1] = i1;
-    g0 *= i0; h0 *= i0; g1 *= i1; h1 *= i1;
-    sm.pgv[2 * lane] = g0;
-    sm.pgv[2 * lane + 1] = g1;
-    sm.phv[2 * lane] = h0;
-    sm.phv[2 * lane + 1] = h1;
-    // the slice's 2x2 Schur complement on (first, last): S = Z^{-1}, Z = [[g0, h0], [g63, h63]]
-    const double z00 = __shfl_sync(0xffffffffu, g0, 0), z0n = __shfl_sync(0xffffffffu, h0, 0);
-    const double zn0 = __shfl_sync(0xffffffffu, g1, 31), znn = __shfl_sync(0xffffffffu, h1, 31);
-    if (lane == 0) {
-      const double id = 1.0 / (z00 * znn - z0n * zn0);
-      sm.pS[0] = znn * id;
-      sm.pS[1] = -z0n * id;
-      sm.pS[2] = -zn0 * id;
-      sm.pS[3] = z00 * id;
-      sm.paf = af;
-      sm.pcl = cl_;
-      for (int q = 0; q < 4; ++q) sm.pe[par][q] = sm.pS[q];
-      sm.pcoup[par][0] = af;
-      sm.pcoup[par][1] = cl_;
-    }
+    r[0] *= sm.pib[2 * lane];
+    r[1] *= sm.pib[2 * lane + 1];
+    double* const out = w == 1 ? sm.pgv : sm.phv;
+    out[2 * lane] = r[0];
+    out[2 * lane + 1] = r[1];
   }
-  cl.sync();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // the slice's 2x2 Schur complement on (first, last): S = Z^{-1}, Z = [[g0, h0], [g63, h63]]
+    const double z00 = sm.pgv[0], z0n = sm.phv[0], zn0 = sm.pgv[63], znn = sm.phv[63];
+    const double id = 1.0 / (z00 * znn - z0n * zn0);
+    sm.pS[0] = znn * id;
+    sm.pS[1] = -z0n * id;
+    sm.pS[2] = -zn0 * id;
+    sm.pS[3] = z00 * id;
+    for (int q = 0; q < 4; ++q) sm.pe[par][q] = sm.pS[q];
+    sm.pcoup[par][0] = sm.paf;
+    sm.pcoup[par][1] = sm.pcl;
+  }
+  f_sync(cl);
   if (w0) {
     // interface rows [F_0, L_0, F_1, L_1, ...]: a_q L_{q-1} + S11 F_q + S12 L_q (F rows),
     // S21 F_q + S22 L_q + c_q F_{q+1} (L rows); PCR multipliers stored per level
@@ -1053,21 +1166,18 @@ __device__ void f_prec_factor(FSmem& sm, cg::cluster_group& cl, const Dev& D, co
       }
     }
     for (int l = 0, st = 1; st < n2; ++l, st <<= 1) {
-      const int il = lane - st, irr = lane + st;
-      const int sl = il >= 0 ? il : 0, sr = irr < n2 ? irr : 0;
-      const double Lb = __shfl_sync(0xffffffffu, ib, sl), La = __shfl_sync(0xffffffffu, ia, sl);
-      const double Lc = __shfl_sync(0xffffffffu, ic, sl);
-      const double Rb = __shfl_sync(0xffffffffu, ib, sr), Ra = __shfl_sync(0xffffffffu, ia, sr);
-      const double Rc = __shfl_sync(0xffffffffu, ic, sr);
-      const bool hl = il >= 0, hr = irr < n2;
+      const double Lb = __shfl_up_sync(0xffffffffu, ib, st), La = __shfl_up_sync(0xffffffffu, ia, st),
+                   Lc = __shfl_up_sync(0xffffffffu, ic, st);
+      const double Rb = __shfl_down_sync(0xffffffffu, ib, st), Ra = __shfl_down_sync(0xffffffffu, ia, st),
+                   Rc = __shfl_down_sync(0xffffffffu, ic, st);
+      const bool hl = lane >= st, hr = lane + st < n2;
       const double k1 = hl ? ia / Lb : 0.0, k2 = hr ? ic / Rb : 0.0;
       if (lane < n2) {
         sm.ik1[l][lane] = k1;
         sm.ik2[l][lane] = k2;
         const double na = hl ? -La * k1 : 0.0, nc = hr ? -Rc * k2 : 0.0;
-        const double nb = ib - (hl ? Lc * k1 : 0.0) - (hr ? Ra * k2 : 0.0);
+        ib = ib - (hl ? Lc * k1 : 0.0) - (hr ? Ra * k2 : 0.0);
         ia = na;
-        ib = nb;
         ic = nc;
       }
     }
@@ -1119,27 +1229,17 @@ __device__ void f_prec(FSmem& sm, cg::cluster_group& cl, const Dev& D, const Ins
     double rc = rhv[6];
 #pragma unroll
     for (int i = 5; i >= 1; --i) rc = rhv[i] - sm.pch[f_pcb(i)][lane] * rc;
-    double r0 = rb[0] - sm.pcs[lane] * rc, r1 = rb[7] - sm.pae[lane] * rhv[6];
-    for (int l = 0, st = 1; st < 64; ++l, st <<= 1) {
-      double nr[2];
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const int i = 2 * lane + p;
-        const double Lr = f_row(r0, r1, i - st), Rr = f_row(r0, r1, i + st);
-        nr[p] = (p ? r1 : r0) - sm.pk1[l][i] * Lr - sm.pk2[l][i] * Rr;
-      }
-      r0 = nr[0];
-      r1 = nr[1];
-    }
-    y0 = r0 * sm.pib[2 * lane];
-    y1 = r1 * sm.pib[2 * lane + 1];
+    double r[2] = {rb[0] - sm.pcs[lane] * rc, rb[7] - sm.pae[lane] * rhv[6]};
+    f_pcr64(sm, r, lane);
+    y0 = r[0];
+    y1 = r[1];
     const double ya = __shfl_sync(0xffffffffu, y0, 0), yb = __shfl_sync(0xffffffffu, y1, 31);
     if (lane == 0) {
       sm.pe[par][4] = sm.pS[0] * ya + sm.pS[1] * yb;
       sm.pe[par][5] = sm.pS[2] * ya + sm.pS[3] * yb;
     }
   }
-  cl.sync();   // every slice's reduced right-hand side published
+  f_sync(cl);   // every slice's reduced right-hand side published
   if (w0) {
     const int Q = G.Q, n2 = 2 * Q;
     double ir = 0.0;
@@ -1264,6 +1364,7 @@ __global__ void __launch_bounds__(kFT, 1) k_pred_fused(Dev D, const int* __restr
   G.N = I.N;
   G.M = I.M;
   G.c0 = (int64_t)G.q * kFS;
+  G.nl = (int)min((int64_t)kFS, (int64_t)I.N - G.c0);
   G.co = I.cell_off;
   const int ii = G.ii;
   const int64_t N = G.N, co = G.co;
@@ -1328,7 +1429,7 @@ __global__ void __launch_bounds__(kFT, 1) k_pred_fused(Dev D, const int* __restr
     {
       // |v0|^2 and |x|^2, and the weighted maximum of v0 (the stopping test), in one pass
       f_reduce<2, true>(
-          sm, cl, par, 2,
+          sm, cl, G.nl, par, 2,
           [&](int i, int c) {
             if (G.c0 + c >= N) return 0.0;
             const double a = i == 0 ? v0[c] : x[G.c0 + c];
@@ -1397,12 +1498,15 @@ __global__ void __launch_bounds__(kFT, 1) k_pred_fused(Dev D, const int* __restr
         // memory.  The second pass also sums |w1|^2, and |w2|^2 = |w1|^2 - |h2|^2 (V
         // orthonormal): exact to rounding while |h2|^2 is small against |w1|^2, which it is
         // after a first pass unless w lies almost in span(V); otherwise a separate sum.
+        // (One pass where it leaves more than a hundredth of w is not enough: P^{-1} C is near
+        // the identity, every step leaves little, and the losses add up to 15% more steps and
+        // 1e-5 in T on the 8192-cell slab.)
         for (int pass = 0; pass < 2; ++pass) {
           const int nd = jc + 1 + pass;   // the dot products, and |w1|^2 in the second pass
           f_reduce<kMaxRestart + 1, false>(
-              sm, cl, par, nd, [&](int i, int c) { return wv[c] * (i <= jc ? Vi(i)[c] : wv[c]); },
+              sm, cl, G.nl, par, nd, [&](int i, int c) { return wv[c] * (i <= jc ? Vi(i)[c] : wv[c]); },
               [](int) { return 0.0; });
-          {
+          if (t < G.nl) {   // (w is 0 past the grid)
             double wj = wv[t];
 #pragma unroll
             for (int i = 0; i < kMaxRestart; ++i) {
@@ -1412,7 +1516,7 @@ __global__ void __launch_bounds__(kFT, 1) k_pred_fused(Dev D, const int* __restr
             wv[t] = wj;
           }
           if (t <= jc) sm.hc[t] = (pass == 0 ? 0.0 : sm.hc[t]) + sm.sums[t];
-          if (pass == 1 && t == 0) {
+          if (pass == 1 && t == 32) {   // (not the warp of the column's update)
             double h2 = 0.0;
             for (int i = 0; i <= jc; ++i) h2 += sm.sums[i] * sm.sums[i];
             const double w1 = sm.sums[jc + 1];
@@ -1428,7 +1532,7 @@ __global__ void __launch_bounds__(kFT, 1) k_pred_fused(Dev D, const int* __restr
           __syncthreads();
         }
         if (sm.sc[2] == 0.0) {
-          f_reduce<1, false>(sm, cl, par, 1, [&](int, int c) { return wv[c] * wv[c]; }, [](int) { return 0.0; });
+          f_reduce<1, false>(sm, cl, G.nl, par, 1, [&](int, int c) { return wv[c] * wv[c]; }, [](int) { return 0.0; });
           if (t == 0) {
             double r, ir;
             f_sqrt_pair(sm.sums[0], r, ir);
