@@ -13,7 +13,7 @@
 // coefficients of V* = max(U*, 0)^{3/4} at the converged iterate, the inflow wall cells
 // keeping F*; for sigma(x) F* itself), read by the Newton kernel.
 //
-// How it runs: one thread-block cluster of Q CTAs per instance (Q in {1,2,4,8,16}), CTA q
+// How it runs: one thread-block cluster of Q = ceil(nx/512) CTAs per instance (1 to 16), CTA q
 // owning the 512-cell slice [512 q, 512 q + 512) (cells past nx are decoupled identity rows).
 // The cluster runs every restart cycle, Arnoldi step, line pass and preconditioner
 // application of the solve without leaving the kernel; control decisions are taken from

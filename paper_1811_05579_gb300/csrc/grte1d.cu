@@ -1422,13 +1422,13 @@ struct grte_ctx {
   long long* d_acc = nullptr;       // Krylov iterations, cycles, iterations run, condition kernels run
   int64_t graph_fixed_launches = 0;
   double tune_ms[3] = {-1.0, -1.0, -1.0};
-  // fused prediction solve: instances grouped by cluster size 1, 2, 4, 8, 16
+  // fused prediction solve: instances grouped by cluster size 1..16
   bool fused = false;
   int* d_finst = nullptr;
-  int fcnt[5] = {0, 0, 0, 0, 0}, foff[5] = {0, 0, 0, 0, 0};
+  int fcnt[17] = {}, foff[17] = {};
   // handles with several cluster sizes: side streams of the smaller ones (fused_solves)
-  cudaStream_t fstream[4] = {nullptr, nullptr, nullptr, nullptr};
-  cudaEvent_t fev_fork = nullptr, fev_join[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaStream_t fstream[15] = {};
+  cudaEvent_t fev_fork = nullptr, fev_join[15] = {};
   cudaEvent_t ev_state = nullptr;   // grte_get_T_device: the caller's stream waits on it
 };
 
@@ -1603,14 +1603,10 @@ static void corr_pass(grte_ctx* h, int dry) {
 }
 
 // ----------------------------------------------------------------------------- fused launches
-// Cluster size of an instance in the fused prediction solve: one 512-cell slice per CTA,
-// rounded up to a power of two (class index 0..4 for 1, 2, 4, 8, 16 CTAs).
-static int fused_class(int64_t nx) {
-  const int64_t q = (nx + kFS - 1) / kFS;
-  int c = 0;
-  while ((1 << c) < q) ++c;
-  return c;
-}
+// Cluster size of an instance in the fused prediction solve: one 512-cell slice per CTA (1 to
+// 16).  Exact, not rounded up to a power of two: CTAs without cells would only hold SMs, and a
+// cluster has to fit into one GPC, which holds two of up to ten CTAs but one of sixteen.
+static int fused_ctas(int64_t nx) { return (int)((nx + kFS - 1) / kFS); }
 
 static bool fused_fits(const Inst& I) { return I.N >= 64 && I.N <= (int64_t)kFQ * kFS && I.M <= 32; }
 
@@ -1665,7 +1661,7 @@ static cudaError_t fused_schedulable(int Qc, int m, bool* ok) {
 static cudaError_t fused_launch(grte_ctx* h, int c, cudaStream_t st) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  fused_config(cfg, at, 1 << c, h->fcnt[c], h->D.m, st);
+  fused_config(cfg, at, c, h->fcnt[c], h->D.m, st);
   return cudaLaunchKernelEx(&cfg, k_pred_fused, h->D, (const int*)(h->d_finst + h->foff[c]));
 }
 
@@ -1675,19 +1671,19 @@ static cudaError_t fused_launch(grte_ctx* h, int c, cudaStream_t st) {
 // fills the chip (at most seven 16-CTA clusters fit, a one-CTA class has one CTA per
 // instance), and in turn each waits for the slowest solve of the one before.  The largest
 // size is launched first: its clusters need the most free SMs at once, and its solves take
-// longest.  64 uneven instances: 2.04 ms of solves per step in turn, 1.10 side by side.
+// longest.  64 uneven instances: 2.04 ms of solves per step in turn, 0.9 side by side.
 // With per-kernel timing on they run in turn, so that each event pair times its launch alone.
 static cudaError_t fused_solves(grte_ctx* h) {
   cudaStream_t st = h->stream;
   cudaError_t e = cudaSuccess;
   if (!h->fev_fork || h->prof_mask != 0) {
-    for (int c = 4; c >= 0 && e == cudaSuccess; --c)
+    for (int c = kFQ; c >= 1 && e == cudaSuccess; --c)
       if (h->fcnt[c]) LAUNCH(GRTE_K_PRED_SOLVE, e = fused_launch(h, c, st));
     return e;
   }
   e = cudaEventRecord(h->fev_fork, st);
   int side = -1;   // the largest size runs on the handle's stream
-  for (int c = 4; c >= 0 && e == cudaSuccess; --c) {
+  for (int c = kFQ; c >= 1 && e == cudaSuccess; --c) {
     if (!h->fcnt[c]) continue;
     cudaStream_t s = side < 0 ? st : h->fstream[side];
     if (side >= 0) e = cudaStreamWaitEvent(s, h->fev_fork, 0);
@@ -2048,18 +2044,18 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
     bool ok = std::all_of(h->inst.begin(), h->inst.end(), [](const Inst& I) { return fused_fits(I); });
     if (ok) CK(fused_attrs());
     ok = ok && fused_smem(m) <= (size_t)g_fused_optin;
-    std::vector<std::vector<int>> cls(5);
+    std::vector<std::vector<int>> cls(kFQ + 1);
     if (ok)
-      for (int i = 0; i < n_inst; ++i) cls[fused_class(h->inst[i].N)].push_back(i);
-    for (int c = 0; c < 5 && ok; ++c) {
+      for (int i = 0; i < n_inst; ++i) cls[fused_ctas(h->inst[i].N)].push_back(i);
+    for (int c = 1; c <= kFQ && ok; ++c) {
       if (cls[c].empty()) continue;
       bool sched = false;
-      CK(fused_schedulable(1 << c, m, &sched));
+      CK(fused_schedulable(c, m, &sched));
       ok = sched;
     }
     if (ok) {
       std::vector<int> order;
-      for (int c = 0; c < 5; ++c) {
+      for (int c = 1; c <= kFQ; ++c) {
         h->foff[c] = (int)order.size();
         h->fcnt[c] = (int)cls[c].size();
         order.insert(order.end(), cls[c].begin(), cls[c].end());
@@ -2067,14 +2063,14 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
       int64_t fd = 0;
       for (int i = 0; i < n_inst; ++i) {
         h->inst[i].fd_off = fd;
-        fd += (int64_t)(1 << fused_class(h->inst[i].N)) * kFS * 32;
+        fd += (int64_t)fused_ctas(h->inst[i].N) * kFS * 32;
       }
       if (dalloc(h, &h->d_finst, n_inst) != cudaSuccess) return nomem("cudaMalloc finst");
       if (dalloc(h, &D.fdata, fd) != cudaSuccess) return nomem("cudaMalloc fdata");
       CK(cudaMemcpy(h->d_finst, order.data(), sizeof(int) * n_inst, cudaMemcpyHostToDevice));
       CK(cudaMemcpy(h->d_inst, h->inst.data(), sizeof(Inst) * n_inst, cudaMemcpyHostToDevice));
       h->fused = true;
-      const int nsize = (int)std::count_if(h->fcnt, h->fcnt + 5, [](int n) { return n > 0; });
+      const int nsize = (int)std::count_if(h->fcnt, h->fcnt + kFQ + 1, [](int n) { return n > 0; });
       for (int i = 0; i + 1 < nsize; ++i) {
         CK(cudaStreamCreateWithFlags(&h->fstream[i], cudaStreamNonBlocking));
         CK(cudaEventCreateWithFlags(&h->fev_join[i], cudaEventDisableTiming));
