@@ -146,7 +146,7 @@ struct Dev {
   void *xb, *S, *F, *Rd, *onode;
   void* S2;        // per element: the correction's e/o flux part (sigma_0/T^3 data passes)
   // preconditioner factors
-  double *pF, *pRd, *pG, *pH, *gw, *pInv;
+  double *pF, *pRd, *pG, *pH, *pInv;
   // GMRES
   double *gx, *gV, *gz, *gH, *gg, *gcs, *gsn, *gbeta, *gxn;
   int *gactive, *gk, *gdone, *gits, *gcycles, *gestconv;
@@ -623,10 +623,20 @@ struct Slice {
   int64_t c0, n;   // this CTA's cells [c0, c0+n) (n = 0 if rank >= nact)
 };
 
+// CTAs that share the N cells of one instance: a lone one up to a cell per thread, above
+// that the whole cluster.  The work on a slice is a chain of short dependent steps, so a
+// CTA takes hardly longer for 128 cells than for 16, and a lone slice needs no cluster
+// barrier, no spikes and no interface system: all Krylov kernels of a 128-cell step took
+// 190 us over 8 slices, 184 over 2 and 165 in one; at 1000 cells 132 us over 8 slices
+// and 137 over 4.
+constexpr int kLoneCells = kTriThreads;
+__host__ __device__ inline int slice_count(int64_t N) {
+  const int64_t half = N / 2;
+  return N <= kLoneCells ? 1 : (int)(half < kCL ? half : kCL);
+}
 __device__ __forceinline__ Slice slice_of(int64_t N, int rank) {
   Slice sl;
-  int64_t half = N / 2;
-  sl.nact = (int)(half < kCL ? half : kCL);
+  sl.nact = slice_count(N);
   if (rank >= sl.nact) { sl.c0 = N; sl.n = 0; return sl; }
   const int64_t base = N / sl.nact, rem = N % sl.nact;
   sl.c0 = rank * base + (rank < rem ? rank : rem);
@@ -636,10 +646,7 @@ __device__ __forceinline__ Slice slice_of(int64_t N, int rank) {
 
 // Reduced-system storage of the preconditioner: kCL slices, each tri_red_size(slice).
 __host__ __device__ inline int64_t prec_red_size(int64_t N) {
-  int64_t half = N / 2;
-  int nact = (int)(half < kCL ? half : kCL);
-  int64_t base = N / nact;
-  return (int64_t)kCL * tri_red_size(base + 1, kTriThreads);
+  return (int64_t)kCL * tri_red_size(N / slice_count(N) + 1, kTriThreads);
 }
 // Factor storage of the preconditioner slices: slice (instance ii, rank) starts at
 // 5 (cell_off + c0 + (ii kCL + rank) kTriThreads), room for tri_fac_size(n, kTriThreads).
@@ -649,19 +656,34 @@ __host__ __device__ inline int64_t prec_fac_off(int64_t cell_off, int64_t c0, in
 
 struct GmresSmem {
   double tri[4 * 2 * kTriThreads];   // reduced system of the slice solves
-  double red[32];
   double part[2][kMaxRestart + 2];   // double-buffered partial sums exchanged by DSMEM
   double ends[6];                    // y_first, y_last, g_first, g_last, h_first, h_last
   double xlr[2];                     // interface values left of and right of this slice
-  double hcol[kMaxRestart + 2];
   double y[kMaxRestart];
-  double gj[2 * kCL][4 * kCL];          // Gauss-Jordan workspace of the interface system
-  double yv[2 * kCL];                   // gathered slice-end values
-  double redm[32][kMaxRestart + 2];     // per-warp partials of a multi-value reduction
+  double prow[2][2 * kCL], pcol[2][2 * kCL];   // pivot row and column of the interface inversion
+  double redm[kTriThreads / 32][kMaxRestart + 2];   // per-warp partials of a reduction
+  double dots[2][kMaxRestart + 2];   // Gram-Schmidt coefficients of the two passes
+  double cs[kMaxRestart], sn[kMaxRestart];     // Givens rotations of the earlier columns
 };
 
-__device__ double cta_sum(double v, double* red) {
+// Barrier over the CTAs that own cells: a lone slice has the instance to itself (the
+// cluster's other CTAs have returned).
+__device__ __forceinline__ void csync(cg::cluster_group& cl, int na) {
+  if (na > 1) cl.sync();
+  else __syncthreads();
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_max(double v) {
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+__device__ double cta_sum(double v, double* red) {
+  v = warp_sum(v);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   __syncthreads();
   if (lane == 0) red[wid] = v;
@@ -671,42 +693,82 @@ __device__ double cta_sum(double v, double* red) {
   return t;
 }
 
-// Sum nv per-CTA partial values over the cluster (fixed rank order).  `buf` selects
-// the half of the double buffer; two consecutive calls must use different halves.
-__device__ void cluster_sums(cg::cluster_group& cl, GmresSmem& sm, int buf, const double* mine, int nv,
-                             double* out) {
-  if (threadIdx.x < nv) sm.part[buf][threadIdx.x] = mine[threadIdx.x];
-  cl.sync();
-  if (threadIdx.x < nv) {
-    double t = 0.0;
-    for (int r = 0; r < kCL; ++r) t += cl.map_shared_rank(&sm.part[buf][0], r)[threadIdx.x];
-    out[threadIdx.x] = t;
+// Combine nv per-CTA values over the cluster in rank order: thread i < nv brings value i,
+// out[i] is the sum, from i = first_max on the maximum.  `buf` selects the half of the
+// double buffer; two consecutive calls must use different halves.
+__device__ __forceinline__ void cluster_combine(cg::cluster_group& cl, int na, GmresSmem& sm, int buf, double mine,
+                                                int nv, int first_max, double* out) {
+  const int i = threadIdx.x;
+  if (na > 1) {
+    if (i < nv) sm.part[buf][i] = mine;
+    cl.sync();
+    if (i < nv) {
+      double v[kCL];
+#pragma unroll
+      for (int r = 0; r < kCL; ++r) v[r] = r < na ? cl.map_shared_rank(&sm.part[buf][0], r)[i] : 0.0;
+      mine = v[0];
+#pragma unroll
+      for (int r = 1; r < kCL; ++r) mine = i >= first_max ? fmax(mine, v[r]) : mine + v[r];
+    }
   }
+  if (i < nv) out[i] = mine;
   __syncthreads();
 }
 
-// Max of nv per-CTA values over the cluster.
-__device__ void cluster_maxs(cg::cluster_group& cl, GmresSmem& sm, int buf, const double* mine, int nv,
-                             double* out) {
-  if (threadIdx.x < nv) sm.part[buf][threadIdx.x] = mine[threadIdx.x];
-  cl.sync();
-  if (threadIdx.x < nv) {
-    double t = 0.0;
-    for (int r = 0; r < kCL; ++r) t = fmax(t, cl.map_shared_rank(&sm.part[buf][0], r)[threadIdx.x]);
-    out[threadIdx.x] = t;
+// dots[i] = w . V_i over the instance, i < nb; with SQ also dots[nb] = w . w.  w: this
+// slice's n values; V: the basis at the slice's first cell, vectors ld apart.
+//
+// Bound: latency (one CTA for up to 256 cells, eight above).  Eight basis vectors at a time, their
+// loads issued together; eight sums cross the warp in 4 + 2 + 1 + 1 + 1 shuffles instead
+// of 40.  Partial sums in K, reductions in double, in a fixed order.
+template <bool SQ, typename K>
+__device__ __forceinline__ void gs_dots(cg::cluster_group& cl, int na, GmresSmem& sm, int buf, const K* w,
+                                        const K* V, int64_t ld, int64_t n, int nb, double* dots) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kTriThreads / 32;
+  const int nwa = n < kTriThreads ? (int)((n + 31) / 32) : nw;   // warps that own cells
+  if (wid < nwa) {
+    K ss = K(0);
+    for (int i0 = 0; i0 < nb; i0 += 8) {
+      K a[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) a[q] = K(0);
+      for (int64_t j = threadIdx.x; j < n; j += kTriThreads) {
+        const K wj = w[j];
+        if (SQ && i0 == 0) ss += wj * wj;
+        K t[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t[q] = i0 + q < nb ? V[(i0 + q) * ld + j] : K(0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a[q] += wj * t[q];
+      }
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = (double)a[q];
+#pragma unroll
+      for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+          const double keep = up ? v[q + h] : v[q], send = up ? v[q] : v[q + h];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+      if ((lane & 3) == 0) sm.redm[wid][i0 + (lane >> 2)] = v[0];   // vector i0 + lane/4
+    }
+    if (SQ) {
+      __syncwarp();
+      const double s = warp_sum((double)ss);
+      if (lane == 0) sm.redm[wid][nb] = s;
+    }
   }
   __syncthreads();
-}
-
-__device__ double cta_max(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
+  const int nv = nb + (SQ ? 1 : 0);
   double t = 0.0;
-  for (int i = 0; i < nw; ++i) t = fmax(t, red[i]);
-  return t;
+  if (threadIdx.x < nv)
+    for (int u = 0; u < nwa; ++u) t += sm.redm[u][threadIdx.x];
+  cluster_combine(cl, na, sm, buf, t, nv, nv, dots);
 }
 
 // z = P^{-1} r on this CTA's slice, P the single-effective-angle Schur operator:
@@ -736,11 +798,17 @@ __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int 
   // the slice's unknowns: shared memory (XS) or the global work vector
   const XAcc<K, XS> wx{XS ? wsm : work + c0};
   const XAcc<K, false> gx{pg + c0}, hx{ph + c0};
+  const int na = sl.nact, m2 = 2 * na;
+  double* inv_rows = D.pInv + ((int64_t)blockIdx.x) * 2 * (2 * kCL);
+  // the interface solve's coefficients (lane: side, column), loaded ahead of their use
+  const int iside = (threadIdx.x >> 4) & 1, icol = threadIdx.x & 15;
+  const bool ilive = threadIdx.x < 32 && icol < m2;
+  double iv = (!FACTOR && na > 1 && ilive) ? inv_rows[iside * 2 * kCL + icol] : 0.0;
   for (int64_t j = threadIdx.x; j < n; j += blockDim.x) wx[j] = ratio_k[c0 + j] * K(r[c0 + j]);
   __syncthreads();
   if (n > 0) {
     tri_solve<FACTOR>(sc, n, wx, F, Rd, red);
-    if (FACTOR) {
+    if (FACTOR && na > 1) {
       for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
         pg[c0 + j] = (j == 0) ? pc.a(c0) : K(0);
         ph[c0 + j] = (j == n - 1) ? pc.c(c0 + n - 1) : K(0);
@@ -749,7 +817,7 @@ __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int 
       tri_solve<false>(sc, n, gx, F, Rd, red);
       tri_solve<false>(sc, n, hx, F, Rd, red);
     }
-    if (threadIdx.x == 0) {
+    if (na > 1 && threadIdx.x == 0) {
       sm.ends[0] = (double)wx[0];
       sm.ends[1] = (double)wx[n - 1];
       sm.ends[2] = (double)pg[c0];
@@ -758,79 +826,57 @@ __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int 
       sm.ends[5] = (double)ph[c0 + n - 1];
     }
   }
-  cl.sync();
-  // interface unknowns X[2q] = u at the first cell of slice q, X[2q+1] = at its last:
-  //   X[2q]   + g_first(q) X[2q-1] + h_first(q) X[2q+2] = y_first(q)
-  //   X[2q+1] + g_last(q)  X[2q-1] + h_last(q)  X[2q+2] = y_last(q)
-  // The matrix depends only on the operator: FACTOR inverts it once per step (one
-  // warp, Gauss-Jordan with partial pivoting) and stores the two rows this slice
-  // needs; every apply is then two short dot products.
-  const int na = sl.nact, m2 = 2 * na;
-  double* inv_rows = D.pInv + ((int64_t)blockIdx.x) * 2 * (2 * kCL);
-  if (FACTOR && threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    const int w2 = 2 * m2;
-    for (int idx = lane; idx < m2 * w2; idx += 32) {
-      const int i = idx / w2, j = idx % w2;
-      sm.gj[i][j] = 0.0;
-    }
-    __syncwarp();
-    if (lane < m2) {
-      const int q = lane / 2, t = lane % 2;
-      const double* e = cl.map_shared_rank(&sm.ends[0], q);
-      sm.gj[lane][lane] = 1.0;
-      if (q > 0) sm.gj[lane][2 * q - 1] += e[2 + t];
-      if (q < na - 1) sm.gj[lane][2 * q + 2] += e[4 + t];
-      sm.gj[lane][m2 + lane] = 1.0;
-    }
-    __syncwarp();
-    for (int col = 0; col < m2; ++col) {
-      int piv = col;
-      if (lane == 0)
-        for (int i = col + 1; i < m2; ++i)
-          if (fabs(sm.gj[i][col]) > fabs(sm.gj[piv][col])) piv = i;
-      piv = __shfl_sync(0xffffffffu, piv, 0);
-      if (piv != col)
-        for (int j = lane; j < w2; j += 32) {
-          const double t = sm.gj[col][j];
-          sm.gj[col][j] = sm.gj[piv][j];
-          sm.gj[piv][j] = t;
-        }
-      __syncwarp();
-      const double ip = 1.0 / sm.gj[col][col];
-      __syncwarp();
-      for (int j = lane; j < w2; j += 32) sm.gj[col][j] *= ip;
-      __syncwarp();
-      double f = (lane < m2 && lane != col) ? sm.gj[lane][col] : 0.0;
-      __syncwarp();
-      for (int i = 0; i < m2; ++i) {
-        const double fi = __shfl_sync(0xffffffffu, f, i);
-        if (i != col && fi != 0.0)
-          for (int j = lane; j < w2; j += 32) sm.gj[i][j] -= fi * sm.gj[col][j];
+  if (na > 1) {
+    cl.sync();
+    // interface unknowns X[2q] = u at the first cell of slice q, X[2q+1] = at its last:
+    //   X[2q]   + g_first(q) X[2q-1] + h_first(q) X[2q+2] = y_first(q)
+    //   X[2q+1] + g_last(q)  X[2q-1] + h_last(q)  X[2q+2] = y_last(q)
+    // The matrix depends only on the operator: FACTOR inverts it once per step and stores
+    // the two rows this slice needs; every apply is then two short dot products.  The
+    // inversion is in place, one element per thread, one barrier per pivot, without row
+    // exchanges: the spikes of a diagonally dominant system have |g| + |h| < 1 in every
+    // row, so the matrix is diagonally dominant too.  (One warp with a pivot search and
+    // the augmented matrix in shared memory took 30 us of a 128-cell step.)
+    if (FACTOR) {
+      static_assert(kTriThreads == (2 * kCL) * (2 * kCL), "one thread per element of the interface matrix");
+      const int i = threadIdx.x / (2 * kCL), c = threadIdx.x % (2 * kCL);
+      double a = i == c ? 1.0 : 0.0;
+      if (i < m2) {
+        const int q = i / 2, t = i % 2;
+        const double* e = cl.map_shared_rank(&sm.ends[0], q);
+        if (q > 0 && c == 2 * q - 1) a += e[2 + t];
+        if (q < na - 1 && c == 2 * q + 2) a += e[4 + t];
       }
-      __syncwarp();
+      for (int p = 0; p < m2; ++p) {
+        const int b = p & 1;
+        if (i == p) sm.prow[b][c] = a;
+        if (c == p) sm.pcol[b][i] = a;
+        __syncthreads();
+        const double ip = 1.0 / sm.prow[b][p];
+        const double rp = (c == p ? 1.0 : sm.prow[b][c]) * ip, f = sm.pcol[b][i];
+        a = i == p ? rp : (c == p ? -f * rp : a - f * rp);
+      }
+      // rows 2 rank - 1 and 2 rank + 2 of the inverse (zero at the ends of the grid)
+      const bool hasL = rank > 0 && rank < na, hasR = rank < na - 1;
+      if (i == (hasL ? 2 * rank - 1 : 0)) inv_rows[c] = hasL ? a : 0.0;
+      if (i == (hasR ? 2 * rank + 2 : 0)) inv_rows[2 * kCL + c] = hasR ? a : 0.0;
+      __syncthreads();
+      if (ilive) iv = inv_rows[iside * 2 * kCL + icol];
     }
-    // rows 2 rank - 1 and 2 rank + 2 of the inverse (columns m2 .. 2 m2 - 1)
-    for (int j = lane; j < m2; j += 32) {
-      inv_rows[j] = (rank > 0 && rank < na) ? sm.gj[2 * rank - 1][m2 + j] : 0.0;
-      inv_rows[2 * kCL + j] = (rank < na - 1) ? sm.gj[2 * rank + 2][m2 + j] : 0.0;
+    if (threadIdx.x < 32) {
+      double acc = ilive ? iv * cl.map_shared_rank(&sm.ends[0], icol >> 1)[icol & 1] : 0.0;
+      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (icol == 0) sm.xlr[iside] = acc;
     }
-  }
-  if (threadIdx.x < m2) {
-    const int q = threadIdx.x / 2, t = threadIdx.x % 2;
-    sm.yv[threadIdx.x] = cl.map_shared_rank(&sm.ends[0], q)[t];
-  }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    double acc = 0.0;
-    const double* row = inv_rows + threadIdx.x * 2 * kCL;
-    for (int j = 0; j < m2; ++j) acc += row[j] * sm.yv[j];
-    sm.xlr[threadIdx.x] = acc;
+  } else if (threadIdx.x < 2) {
+    sm.xlr[threadIdx.x] = 0.0;
   }
   __syncthreads();
   const K ul = K(sm.xlr[0]), ur = K(sm.xlr[1]);
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) wx[j] = wx[j] - ul * pg[c0 + j] - ur * ph[c0 + j];
-  __syncthreads();
+  if (na > 1) {
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) wx[j] = wx[j] - ul * pg[c0 + j] - ur * ph[c0 + j];
+    __syncthreads();
+  }
   const K wv2 = K(I.wv2), wv = K(I.wv);
   for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
     const int64_t g = c0 + j;
@@ -847,8 +893,8 @@ __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int 
 // per-angle e/o parts, 16 loads issued together, four partial sums (type A) combined
 // in a fixed order; the two inflow wall cells sum their double wall fluxes.
 template <typename R, typename A = R>
-__device__ __forceinline__ A eo_sum(const Dev& D, const Inst& I, int64_t j) {
-  const R* S = (const R*)D.S + I.elem_off + j;
+__device__ __forceinline__ A eo_sum(const void* parts, const Inst& I, int64_t j) {
+  const R* S = (const R*)parts + I.elem_off + j;
   const int64_t N = I.N;
   A p[4] = {A(0), A(0), A(0), A(0)};
   int k = 0;
@@ -879,14 +925,14 @@ template <typename R>
 __device__ __forceinline__ double flux_sum(const Dev& D, const Inst& I, int64_t j) {
   const double fr = D.Frho[I.cell_off + j];
   if (wall_cell(I, j)) return fr + wall_sum(D, I, j);
-  return fr + eo_sum<R, double>(D, I, j);
+  return fr + eo_sum<R, double>(D.S, I, j);
 }
 
 // in the bulk type (Krylov directions)
 template <typename R>
 __device__ __forceinline__ R flux_sum_k(const Dev& D, const Inst& I, int64_t j) {
   if (wall_cell(I, j)) return R(D.Frho[I.cell_off + j] + wall_sum(D, I, j));
-  return pick<R>(D.Frho, D.fc.Frho)[I.cell_off + j] + eo_sum<R>(D, I, j);
+  return pick<R>(D.Frho, D.fc.Frho)[I.cell_off + j] + eo_sum<R>(D.S, I, j);
 }
 
 // The correction's flux at a cell j that is not an inflow wall cell (sigma_0/T^3, the
@@ -901,15 +947,17 @@ __device__ __forceinline__ double corr_flux_sum(const Dev& D, const Inst& I, int
   const double xj = x[j], xl = j > 0 ? x[j - 1] : 0.0, xr = j < N - 1 ? x[j + 1] : 0.0;
   const double dR = j < N - 1 ? D.cf.dsx[co + j + 1] : 0.0, dL = D.cf.dsx[co + j];
   const double f = I.wv2 * (dR * (xj - xr) + dL * (xj - xl));
-  const R* S = (const R*)D.S2 + I.elem_off + j;
-  double acc = 0.0;
-  for (int k = 0; k < I.M; ++k) acc += (double)S[(int64_t)k * N];
-  return f + acc;
+  return f + eo_sum<R, double>(D.S2, I, j);
 }
 
 enum { G_RESTART_FIRST = 0, G_RESTART = 1, G_ARNOLDI = 2, G_UPDATE = 3 };
 
 
+// Bound: latency, chains of dependent binary64 steps and loads on few cells per CTA.  So the
+// loads of a chain go out ahead of it (basis vectors by eight, factors, rotations, H),
+// values cross a warp or the cluster together, and there are as few barriers as the
+// algorithm needs.  All Krylov kernels of a step: 128 cells 265 -> 166 us, 1000 cells
+// 177 -> 133, 8192 cells (binary64 rate of the eight SMs) 906 -> 863.
 // GMRES bookkeeping, one cluster per instance (restart length m, left
 // preconditioned).  Vectors live in global memory: x (iterate), V[0..m] (Krylov
 // basis), z (scratch).  Scalars (H, g, Givens) are computed identically by every
@@ -929,13 +977,15 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
   const int64_t N = I.N, co = I.cell_off;
   const Slice sl = slice_of(N, rank);
   const int64_t c0 = sl.c0, n = sl.n;
-  const int m = D.m;
+  const int m = D.m, na = sl.nact;
+  if (na == 1 && rank > 0) return;   // a lone slice: no cluster barrier below
   double* x = D.gx + co;           // iterate, double
   double* zd = D.gz + co;          // scratch as double (residual) ...
   K* zk = (K*)D.gz + co;           // ... or as K (a preconditioner input)
   K* work = (K*)D.gwork + co;
   const int64_t ncell_tot = D.gz - D.gx;     // gz = gx + ncell_total (allocation layout)
-  auto Vi = [&](int i) { return (K*)D.gV + (int64_t)i * ncell_tot + co; };
+  K* const V = (K*)D.gV + co;
+  auto Vi = [&](int i) { return V + (int64_t)i * ncell_tot; };
   double* H = D.gH + (int64_t)ii * (kMaxRestart + 1) * kMaxRestart;
   double* g = D.gg + (int64_t)ii * (kMaxRestart + 1);
   double* cs = D.gcs + (int64_t)ii * kMaxRestart;
@@ -950,45 +1000,58 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
     const int cycles_prev = D.gcycles[ii];
     // r = -R(x) from the FULL pass that just ran at x
     double* r = zd;
+    double xm = 0.0;
     for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) {
       const double fl = flux_sum<R>(D, I, j);
-      const double Rj = alpha[j] * x[j] - kcd[j] * D.rho_n[co + j] - sac[j] * D.U[co + j] + kdx[j] * fl;
+      const double xj = x[j];
+      const double Rj = alpha[j] * xj - kcd[j] * D.rho_n[co + j] - sac[j] * D.U[co + j] + kdx[j] * fl;
       r[j] = -Rj;
       D.Fs[co + j] = fl;                    // F* of the current iterate (final at convergence)
       D.Fc[co + j] = (I.kind == GRTE_SIGMA_T3 && !wall_cell(I, j)) ? corr_flux_sum<R>(D, I, j, x) : fl;
+      xm = fmax(xm, fabs(xj));
     }
-    // per-cell weights of the stopping test: the preconditioned residual relative to
-    // |x_j| (floor wfloor max|x|: 1e-13 in FP64, 1e-8 with binary32 line solves), so
-    // that the test bounds every cell's relative correction and not only the large
-    // cells' share of a 2-norm
-    double xm = 0.0;
-    for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) xm = fmax(xm, fabs(x[j]));
-    xm = cta_max(xm, sm.red);
-    __shared__ double xms[1];
-    cluster_maxs(cl, sm, 0, &xm, 1, xms);
-    for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x)
-      D.gw[co + j] = 1.0 / (fabs(x[j]) + D.wfloor * xms[0] + 1e-300);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    xm = warp_max(xm);
+    if (lane == 0) sm.redm[wid][0] = xm;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int u = 1; u < nw; ++u) xm = fmax(xm, sm.redm[u][0]);
+      sm.part[0][0] = xm;   // read after the barriers of the preconditioner
+    }
     __syncthreads();
     K* v0 = Vi(0);
     if (MODE == G_RESTART_FIRST) prec_apply_cl<true, XS, K, double>(D, I, sl, rank, cl, r, v0, work, wsm, sm);
     else prec_apply_cl<false, XS, K, double>(D, I, sl, rank, cl, r, v0, work, wsm, sm);
+    double xmax = 0.0;
+    for (int q = 0; q < na; ++q)
+      xmax = fmax(xmax, na > 1 ? cl.map_shared_rank(&sm.part[0][0], q)[0] : sm.part[0][0]);
+    // per-cell weights of the stopping test: the preconditioned residual relative to
+    // |x_j| (floor wfloor max|x|: 1e-13 in FP64, 1e-8 with binary32 line solves), so
+    // that the test bounds every cell's relative correction and not only the large
+    // cells' share of a 2-norm
+    const double wfl = D.wfloor * xmax + 1e-300;
     double loc[3] = {0.0, 0.0, 0.0};
     K ss = K(0);
     for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) {
       const K vj = v0[j];
       ss += vj * vj;
       loc[1] += x[j] * x[j];
-      loc[2] = fmax(loc[2], fabs((double)vj) * D.gw[co + j]);
+      loc[2] = fmax(loc[2], fabs((double)vj) / (fabs(x[j]) + wfl));
     }
-    loc[0] = (double)ss;
-    loc[0] = cta_sum(loc[0], sm.red);
-    loc[1] = cta_sum(loc[1], sm.red);
-    loc[2] = cta_max(loc[2], sm.red);
-    __shared__ double tots[2], tmax[1];
-    cluster_sums(cl, sm, 1, loc, 2, tots);
-    cluster_maxs(cl, sm, 0, loc + 2, 1, tmax);
+    loc[0] = warp_sum((double)ss);
+    loc[1] = warp_sum(loc[1]);
+    loc[2] = warp_max(loc[2]);
+    if (lane == 0)
+      for (int q = 0; q < 3; ++q) sm.redm[wid][q] = loc[q];
+    __syncthreads();
+    double mine = 0.0;
+    if (threadIdx.x < 3)
+      for (int u = 0; u < nw; ++u)
+        mine = threadIdx.x == 2 ? fmax(mine, sm.redm[u][2]) : mine + sm.redm[u][threadIdx.x];
+    double* tots = sm.dots[0];   // |v|^2, |x|^2, the largest weighted |v_j|
+    cluster_combine(cl, na, sm, 1, mine, 3, 2, tots);
     const double nrm = sqrt(tots[0]), xn = sqrt(tots[1]);
-    const double rinf = tmax[0];
+    const double rinf = tots[2];
     // Converged when every cell's relative preconditioned correction is below rtol.
     // Restarted GMRES cannot go below the rounding floor of the residual evaluation
     // itself (a sum of terms much larger than the residual): a restart cycle that
@@ -1017,7 +1080,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
       const K inv = K(1.0 / nrm);
       for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) v0[j] *= inv;
     }
-    cl.sync();   // no CTA leaves while another may still read its shared memory
+    csync(cl, na);   // no CTA leaves while another may still read its shared memory
     // per-cell parts of the first direction pass (V_0 of the neighbouring slices is
     // complete after the cluster barrier)
     // (FP64 mode only: in the mixed mode the per-cell kernel runs on all SMs instead,
@@ -1032,7 +1095,11 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
     // g[jcol] is rotated by rank 0 at the end of this step: read it now, before the
     // cluster barriers below, so that no CTA can see the rotated value and every CTA
     // takes the same continue/stop decision
-    const double g_jcol = g[jcol];
+    const double g_jcol = g[jcol], xn = D.gxn[ii];
+    if (threadIdx.x < jcol) {
+      sm.cs[threadIdx.x] = cs[threadIdx.x];
+      sm.sn[threadIdx.x] = sn[threadIdx.x];
+    }
     // C v_j = alpha v_j + kappa/dx * sum_k S_k  (the HOM pass just ran on v_j)
     const K* vj = Vi(jcol);
     K* cv = zk;
@@ -1042,82 +1109,69 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
     __syncthreads();
     K* wv = Vi(jcol + 1);
     prec_apply_cl<false, XS, K, K>(D, I, sl, rank, cl, cv, wv, work, wsm, sm);
-    // classical Gram-Schmidt, twice (CGS2): two cluster reductions instead of j+1
-    __shared__ double dots[kMaxRestart + 2];
-    __shared__ double hc[kMaxRestart + 2];   // Hessenberg column (thread 0 finishes it)
+    // classical Gram-Schmidt, twice (CGS2), w in shared memory (XS): each thread works on
+    // its own cells only.  The second pass's reduction also carries |w|^2, from which the
+    // norm after it is |w|^2 - sum_i d_i^2 (its coefficients d_i are rounding-level, so
+    // nothing cancels unless w lies in the basis, where the cycle ends).
+    const int nb = jcol + 1;
+    K* w = XS ? wsm : wv + c0;
+    if (XS)
+      for (int64_t j = threadIdx.x; j < n; j += blockDim.x) w[j] = wv[c0 + j];
+    gs_dots<false>(cl, na, sm, 0, w, V + c0, ncell_tot, n, nb, sm.dots[0]);
+    auto gs_sub = [&](const double* d, double scale, K* out) {
+      for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        K t = w[j];
+        for (int i0 = 0; i0 < nb; i0 += 8) {
+          K b[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) b[q] = i0 + q < nb ? V[(i0 + q) * ncell_tot + c0 + j] : K(0);
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (i0 + q < nb) t -= K(d[i0 + q]) * b[q];
+        }
+        out[j] = t * K(scale);
+      }
+    };
+    gs_sub(sm.dots[0], 1.0, w);
+    gs_dots<true>(cl, na, sm, 1, w, V + c0, ncell_tot, n, nb, sm.dots[1]);
+    double nn = sm.dots[1][nb];
+    for (int i = 0; i < nb; ++i) nn -= sm.dots[1][i] * sm.dots[1][i];
+    const double inrm = nn > 0.0 ? rsqrt(nn) : 0.0;
+    const double nrm = nn > 0.0 ? nn * inrm : (nn <= 0.0 ? 0.0 : nn);   // NaN stays NaN
     __shared__ int cont_s;                   // 1: another Arnoldi step follows
-    if (threadIdx.x <= jcol + 1) hc[threadIdx.x] = 0.0;
-    for (int pass = 0; pass < 2; ++pass) {
-      // all jcol+1 dot products in one sweep and one CTA reduction
-      // per-thread partial sums in K, reductions in double
-      K lk[kMaxRestart + 1];
-      double loc[kMaxRestart + 1];
-      for (int i = 0; i <= jcol; ++i) lk[i] = K(0);
-      for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) {
-        const K wj = wv[j];
-        for (int i = 0; i <= jcol; ++i) lk[i] += wj * Vi(i)[j];
+    if (threadIdx.x == blockDim.x - 32) {    // the last warp: the one with the fewest cells
+      // Hessenberg column: the earlier rotations (one fused multiply-add each on the
+      // serial chain), then the new one
+      double a0 = sm.dots[0][0] + sm.dots[1][0];
+      for (int i = 0; i < jcol; ++i) {
+        const double hi = sm.dots[0][i + 1] + sm.dots[1][i + 1];
+        const double t = sm.cs[i] * a0 + sm.sn[i] * hi;
+        a0 = sm.cs[i] * hi - sm.sn[i] * a0;
+        if (rank == 0) H[i * kMaxRestart + jcol] = t;
       }
-      const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-      for (int i = 0; i <= jcol; ++i) {
-        double v = (double)lk[i];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sm.redm[wid][i] = v;
-      }
-      __syncthreads();
-      for (int i = 0; i <= jcol; ++i) {
-        double t = 0.0;
-        for (int w = 0; w < nw; ++w) t += sm.redm[w][i];   // same order in every thread
-        loc[i] = t;
-      }
-      __syncthreads();
-      cluster_sums(cl, sm, pass, loc, jcol + 1, dots);
-      for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) {
-        K t = wv[j];
-        for (int i = 0; i <= jcol; ++i) t -= K(dots[i]) * Vi(i)[j];
-        wv[j] = t;
-      }
-      if (threadIdx.x <= jcol) hc[threadIdx.x] += dots[threadIdx.x];
-      __syncthreads();
-    }
-    K l1 = K(0);
-    for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) l1 += wv[j] * wv[j];
-    double loc1 = cta_sum((double)l1, sm.red);
-    __shared__ double nn[1];
-    cluster_sums(cl, sm, 0, &loc1, 1, nn);
-    const double nrm = sqrt(nn[0]);
-    if (threadIdx.x == 0) {
-      hc[jcol + 1] = nrm;
-      for (int i = 0; i < jcol; ++i) {           // previous Givens rotations
-        const double t = cs[i] * hc[i] + sn[i] * hc[i + 1];
-        hc[i + 1] = -sn[i] * hc[i] + cs[i] * hc[i + 1];
-        hc[i] = t;
-      }
-      const double a0 = hc[jcol], b0 = hc[jcol + 1];
-      const double rr = hypot(a0, b0);
-      const double c0g = rr > 0.0 ? a0 / rr : 1.0, s0g = rr > 0.0 ? b0 / rr : 0.0;
-      hc[jcol] = rr;
-      const double gj = g_jcol;
-      const double gnext = -s0g * gj;
+      // (hypot and divisions, correctly rounded: they run beside the other warps' sweep)
+      const double rr = hypot(a0, nrm);
+      const double c0g = rr > 0.0 ? a0 / rr : 1.0, s0g = rr > 0.0 ? nrm / rr : 0.0;
+      const double gnext = -s0g * g_jcol;
       // GMRES's own (2-norm) estimate; the per-cell test runs on the true residual.
       // Every CTA takes the same decision (its inputs are cluster-wide values).
-      const bool est = fabs(gnext) <= 0.05 * D.rtol * D.gxn[ii];
+      const bool est = fabs(gnext) <= 0.05 * D.rtol * xn;
       const bool stop = est || nrm == 0.0 || jcol + 1 >= m;
       cont_s = stop ? 0 : 1;
       if (rank == 0) {
+        H[jcol * kMaxRestart + jcol] = rr;
         cs[jcol] = c0g;
         sn[jcol] = s0g;
         g[jcol + 1] = gnext;
-        g[jcol] = c0g * gj;
-        for (int i = 0; i <= jcol; ++i) H[i * kMaxRestart + jcol] = hc[i];
+        g[jcol] = c0g * g_jcol;
         D.gk[ii] = jcol + 1;
         D.gits[ii] += 1;
         if (est) D.gestconv[ii] = 1;
         if (stop) D.gactive[ii] = 0;
       }
     }
-    const K inv = K(nrm > 0.0 ? 1.0 / nrm : 0.0);
-    for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) wv[j] *= inv;
-    cl.sync();
+    gs_sub(sm.dots[1], inrm, wv + c0);
+    csync(cl, na);
     // per-cell parts of the next direction pass (V_{j+1} complete after the barrier)
     if (FUSED_PARTS && cont_s)
       for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) cellpart_cell<K>(D, I, co + j, j, wv, 0);
@@ -1127,21 +1181,39 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
   if (MODE == G_UPDATE) {
     if (D.gdone[ii]) return;
     const int kk = D.gk[ii];
-    if (threadIdx.x == 0) {
-      for (int i = kk - 1; i >= 0; --i) {
-        double t = g[i];
-        for (int l = i + 1; l < kk; ++l) t -= H[i * kMaxRestart + l] * sm.y[l];
-        sm.y[i] = t / H[i * kMaxRestart + i];
+    if (threadIdx.x < 32) {
+      // H y = g, lane l holding row l: the loads go out together, the divisions run side by
+      // side, and the chain is a multiplication, a shuffle and a multiply-add per unknown
+      static_assert(kMaxRestart <= 32, "one lane per row");
+      const int l = threadIdx.x;
+      double hr[kMaxRestart];
+#pragma unroll
+      for (int i = 0; i < kMaxRestart; ++i) hr[i] = (l < i && i < kk) ? H[l * kMaxRestart + i] : 0.0;
+      double gl = l < kk ? g[l] : 0.0;
+      const double ih = l < kk ? 1.0 / H[l * kMaxRestart + l] : 0.0;
+#pragma unroll
+      for (int i = kMaxRestart - 1; i >= 0; --i) {
+        if (i >= kk) continue;
+        const double yi = __shfl_sync(0xffffffffu, gl * ih, i);
+        if (l < i) gl -= hr[i] * yi;
       }
+      if (l < kk) sm.y[l] = gl * ih;
     }
     __syncthreads();
     for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) {
       double t = x[j];
-      for (int i = 0; i < kk; ++i) t += sm.y[i] * (double)Vi(i)[j];
+      for (int i0 = 0; i0 < kk; i0 += 8) {
+        double b[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) b[q] = i0 + q < kk ? (double)Vi(i0 + q)[j] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (i0 + q < kk) t += sm.y[i0 + q] * b[q];
+      }
       x[j] = t;
     }
     if (FUSED_PARTS) {
-      cl.sync();
+      csync(cl, na);
       // per-cell parts of the data pass at the updated iterate
       for (int64_t j = c0 + threadIdx.x; j < c0 + n; j += blockDim.x) cellpart_cell<double>(D, I, co + j, j, x, 1);
     }
@@ -1911,8 +1983,7 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
     }
     h->maxN = std::max<int64_t>(h->maxN, p.nx);
     {
-      const int64_t nact = std::min<int64_t>(p.nx / 2, kCL);
-      h->max_slice = std::max<int64_t>(h->max_slice, p.nx / nact + 1);
+      h->max_slice = std::max<int64_t>(h->max_slice, p.nx / slice_count(p.nx) + 1);
     }
     poff += prec_red_size(p.nx);
     coff += p.nx;
@@ -1988,7 +2059,7 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
     if (dalloc(h, &p_, es * h->nred) != cudaSuccess) return nomem("cudaMalloc Rd"); D.Rd = p_;
     if (dalloc(h, &p_, es * nn) != cudaSuccess) return nomem("cudaMalloc onode"); D.onode = p_;
   }
-  AL(D.pF, 5 * (nc + (int64_t)n_inst * kCL * kTriThreads)); AL(D.pRd, h->npred); AL(D.pG, nc); AL(D.pH, nc); AL(D.gw, nc);
+  AL(D.pF, 5 * (nc + (int64_t)n_inst * kCL * kTriThreads)); AL(D.pRd, h->npred); AL(D.pG, nc); AL(D.pH, nc);
   AL(D.pInv, (int64_t)n_inst * kCL * 2 * (2 * kCL));
   // x, z contiguous so that the GMRES kernel can recover the total cell count
   double* xz = nullptr;
@@ -3008,7 +3079,7 @@ constexpr int64_t kNaMaxCells = 4096;
 constexpr int kNaMaxAngles = 32;
 constexpr int64_t kNaMaxElems = 65536;                      // nx * n_angle
 constexpr int64_t kNaMaxNodeElems = kNaMaxElems + kNaMaxAngles;
-constexpr int64_t kNaCellArrays = 42;                       // per-cell double arrays (40 + the x/z pair)
+constexpr int64_t kNaCellArrays = 41;                       // per-cell double arrays (39 + the x/z pair)
 constexpr int64_t kNaAlign = 256;
 __host__ __device__ constexpr int64_t na_round(int64_t b) { return (b + kNaAlign - 1) / kNaAlign * kNaAlign; }
 // line solves run at kTriThreads threads here: per line at most 2 kTriThreads reduced
@@ -3029,11 +3100,11 @@ constexpr int64_t kNaBytes =
     na_round(4 * 16) + na_round(sizeof(Inst)) + na_round(sizeof(Line) * kNaMaxAngles) + na_round(8);
 }  // namespace grte
 
-// Work memory of grte_step1d_noalloc: kNaBytes = 11,198,464 bytes (about 11.2 MB),
+// Work memory of grte_step1d_noalloc: kNaBytes = 11,165,696 bytes (about 11.2 MB),
 // held by every GPU that loads the library until the process exits.  Calls share it
 // (see include/grte.h, which states the same figure; the assertion keeps the two in
 // step when the layout changes).
-static_assert(grte::kNaBytes == 11198464, "no-alloc work memory size changed: update the documented figure");
+static_assert(grte::kNaBytes == 11165696, "no-alloc work memory size changed: update the documented figure");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[grte::kNaBytes];
 static void* g_noalloc_base[64];   // device address of g_noalloc_scratch, per device
 
@@ -3158,7 +3229,7 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
                                    &D.P3, &D.Frho, &D.gU, &D.Q1, &D.Q2, &D.gwork, &D.cf.kc, &D.cf.s,
                                    &D.cf.alpha, &D.cf.A, &D.cf.gam, &D.cf.gl, &D.cf.gu, &D.cf.gb, &D.cf.dl,
                                    &D.cf.od, &D.cf.dlx, &D.cf.kcd, &D.cf.kdx, &D.cf.sac, &D.cf.ralpha,
-                                   &D.cf.ratio, &D.cf.fR, &D.cf.fL, &D.cf.gbx, &D.pG, &D.pH, &D.gw,
+                                   &D.cf.ratio, &D.cf.fR, &D.cf.fL, &D.cf.gbx, &D.pG, &D.pH,
                                    &D.cf.dsx, &D.cf.ods, &D.Fc};
   for (int i = 0; i < kNaCellArrays - 2; ++i) *cells[i] = (double*)take(8 * kNaMaxCells);
   // x and z of the Krylov kernels are adjacent: the kernels take the cell stride of
@@ -3244,7 +3315,7 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
   if (line_kernel_attrs() != cudaSuccess) { ctx.h_flags = nullptr; return GRTE_ECUDA; }
   ctx.maxN = N;
   ctx.xs = line_fits(&ctx, kTriThreads);
-  ctx.max_slice = N / std::min<int64_t>(N / 2, kCL) + 1;
+  ctx.max_slice = N / slice_count(N) + 1;
   ctx.gxs = (tri_xs_len(ctx.max_slice) * 8 + 15) / 16 * 16 <= g_gmres_dyn;
   ctx.nt = kTriThreads;
   for (int64_t n = 0; n < nsteps; ++n) {
