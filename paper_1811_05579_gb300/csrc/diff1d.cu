@@ -49,17 +49,6 @@ struct DDev {
   int* status;
 };
 
-// 1/b: the binary32 reciprocal r and the third-order residual correction r (1 + e + e^2),
-// e = 1 - b r < 2^-22 (three binary64 operations instead of the divide sequence); outside
-// the binary32 range the division.
-__device__ __forceinline__ double d_rcp(double b) {
-  const float f = (float)b;
-  if (!(fabsf(f) > 1e-30f && fabsf(f) < 1e30f)) return 1.0 / b;
-  const double r = (double)__frcp_rn(f);
-  const double e = fma(-b, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // u^{3/4} for u >= 0 as u u^{-1/4}: r = u^{-1/4} from binary32 and one third-order step,
 // r (1-e)^{-1/4} = r (1 + e/4 + 5 e^2/32 + ...), e = 1 - u r^4 < 2^-19; outside the
 // binary32 range the library power.
@@ -227,13 +216,13 @@ struct DSmem {
 struct DChunk { double rc[3], cc[3], ac[3]; };
 __device__ __forceinline__ void d_eliminate(const double* a, const double* b, const double* c, const double* r,
                                             DChunk& k, double& A, double& B, double& R) {
-  double inv = d_rcp(b[0]);
+  double inv = rcp64(b[0]);
   k.ac[0] = a[0] * inv;
   k.cc[0] = c[0] * inv;
   k.rc[0] = r[0] * inv;
 #pragma unroll
   for (int u = 1; u < 3; ++u) {
-    inv = d_rcp(fma(-a[u], k.cc[u - 1], b[u]));
+    inv = rcp64(fma(-a[u], k.cc[u - 1], b[u]));
     k.ac[u] = -a[u] * k.ac[u - 1] * inv;
     k.cc[u] = c[u] * inv;
     k.rc[u] = fma(-a[u], k.rc[u - 1], r[u]) * inv;
@@ -270,7 +259,7 @@ __device__ __forceinline__ void d_pcr(int lane, int n, double& a, double& c, dou
       r = fma(-c, rR, r);
       cn = -c * cR;
     }
-    const double inv = d_rcp(b);
+    const double inv = rcp64(b);
     a = an * inv;
     c = cn * inv;
     r *= inv;
@@ -383,7 +372,7 @@ __global__ void __launch_bounds__(kFT) k_diff(DDev D, int first, int Q, int nste
       const double m0 = __shfl_down_sync(~0u, kb.rc[0], 1), m1 = __shfl_down_sync(~0u, kb.cc[0], 1),
                    m2 = __shfl_down_sync(~0u, kb.ac[0], 1);
       if (lane < 31) {   // lane 31's separator is the CTA's: its row stays as it is
-        const double inv = d_rcp(fma(-c[3], m2, B));
+        const double inv = rcp64(fma(-c[3], m2, B));
         la = A * inv;
         lc = -c[3] * m1 * inv;
         lr = fma(-c[3], m0, R) * inv;
@@ -426,7 +415,7 @@ __global__ void __launch_bounds__(kFT) k_diff(DDev D, int first, int Q, int nste
             r = fma(-x, f0, r);
           }
         }
-        const double inv = d_rcp(b);
+        const double inv = rcp64(b);
         a *= inv;
         c *= inv;
         r *= inv;
@@ -438,7 +427,7 @@ __global__ void __launch_bounds__(kFT) k_diff(DDev D, int first, int Q, int nste
         if (q == 0) SL = 0.0;
         if (lane == 0) sm.nxt = q < Q - 1 ? nx : 0.0;
       } else {
-        S = sm.pub[5] * d_rcp(sm.pub[4]);
+        S = sm.pub[5] * rcp64(sm.pub[4]);
         if (lane == 0) sm.nxt = 0.0;
       }
       const double s = lane < 31 ? lr - la * SL - lc * S : S;

@@ -1446,7 +1446,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_corr_line(Dev D, int dry) {
   R* on = (R*)D.onode + oo;
   const double *dlx = D.cf.dlx + co, *kcd = D.cf.kcd + co, *kdx = D.cf.kdx + co, *Q1 = D.Q1 + co,
                *Q2 = D.Q2 + co, *gU = D.gU + co;
-  const double two_eps = I.two_eps, inv_eps = I.inv_eps;
+  const double two_eps = I.two_eps, inv_eps = I.inv_eps, vie = v * inv_eps;
   const R vr = R(v), v2r = R(v * v);
   constexpr bool F32 = sizeof(R) == 4;
   const R* odr = pick<R>(D.cf.od, D.fc.od) + co;
@@ -1462,8 +1462,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_corr_line(Dev D, int dry) {
         const R ke = (R)D.fc.kdxe[g];
         xb[j] = D.fc.Q1[g] + D.fc.kcde[g] * Eh[j] - ke * vr * (on[j + 1] - on[j]) + ke * v2r * D.fc.Q2[g];
       } else {
-        xb[j] = R(Q1[j]) + R(kcd[j] * inv_eps) * Eh[j] - R(kdx[j] * v * inv_eps) * (on[j + 1] - on[j]) +
-                R(kdx[j] * v * v * inv_eps) * R(Q2[j]);
+        // the per-line factors first: six binary64 operations instead of eleven
+        xb[j] = Q1[j] + kcd[j] * (inv_eps * Eh[j]) + kdx[j] * (vie * (v * Q2[j] - (on[j + 1] - on[j])));
       }
     } else {
       double Dj;
@@ -1482,7 +1482,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_corr_line(Dev D, int dry) {
   for (int64_t i = threadIdx.x; i <= N; i += NT) {
     auto Oint = [&](int64_t n) -> R {
       if constexpr (F32) return on[n] - vr * D.fc.gU[co + n] - D.fc.dlxe[co + n] * vr * (xb[n] - xb[n - 1]);
-      else return on[n] - vr * R(gU[n]) - R(dlx[n] * eps) * vr * (xb[n] - xb[n - 1]);
+      else return on[n] - v * (gU[n] + dlx[n] * (eps * (xb[n] - xb[n - 1])));
     };
     R Oi;
     if (i >= 1 && i <= N - 1) Oi = Oint(i);
