@@ -161,6 +161,7 @@ struct Dev {
   float* fdata;     // fused solve: data terms of the prediction, [slice cell][32 angles]
   int use_guess, log_samples;
   int start_prev;   // 1: Newton starts one step from T^n instead of the closed-form bound
+  int ncl;  // CTAs per cluster of the Krylov kernels
   int m;  // restart length
   int maxcycles;  // restart cycles per step before ENONCONV
   double rtol, stall, wfloor;
@@ -608,12 +609,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_pred_line(Dev D, const void* 
 }
 
 // ----------------------------------------------------------------------------- instance (GMRES)
-// The per-instance Krylov work runs on a thread-block cluster of kCL CTAs: each CTA
+// The per-instance Krylov work runs on a thread-block cluster of ncl CTAs (8, or 16 for few
+// large FP64 instances: gmres_cluster): each CTA
 // owns a contiguous slice of the instance's cells; dot products are reduced through
 // distributed shared memory (fixed rank order, so every CTA gets the same value);
 // the preconditioner's tridiagonal solve is partitioned across the cluster by the
-// spike method (local solves plus a 2*kCL interface system).
-constexpr int kCL = 8;
+// spike method (local solves plus a 2 ncl interface system).
+constexpr int kCL = 8, kCLMax = 16;
 
 template <typename K>
 struct PrecCoef {  // A + (A/alpha) (wv2 Gint + wv Gbdry), evaluated in double, stored in K
@@ -647,28 +649,26 @@ struct Slice {
 // 190 us over 8 slices, 184 over 2 and 165 in one; at 1000 cells 132 us over 8 slices
 // and 137 over 4.
 constexpr int kLoneCells = kTriThreads;
-__host__ __device__ inline int slice_count(int64_t N) {
-  const int64_t half = N / 2;
-  return N <= kLoneCells ? 1 : (int)(half < kCL ? half : kCL);
-}
+__host__ __device__ inline int slice_count(int64_t N, int ncl) { return N <= kLoneCells ? 1 : ncl; }
+template <int CL>
 __device__ __forceinline__ Slice slice_of(int64_t N, int rank) {
   Slice sl;
-  sl.nact = slice_count(N);
+  sl.nact = slice_count(N, CL);
   if (rank >= sl.nact) { sl.c0 = N; sl.n = 0; return sl; }
-  const int64_t base = N / sl.nact, rem = N % sl.nact;
+  const int64_t base = sl.nact == 1 ? N : N / CL, rem = sl.nact == 1 ? 0 : N % CL;
   sl.c0 = rank * base + (rank < rem ? rank : rem);
   sl.n = base + (rank < rem ? 1 : 0);
   return sl;
 }
 
-// Reduced-system storage of the preconditioner: kCL slices, each tri_red_size(slice).
-__host__ __device__ inline int64_t prec_red_size(int64_t N) {
-  return (int64_t)kCL * tri_red_size(N / slice_count(N) + 1, kTriThreads);
+// Reduced-system storage of one slice of the preconditioner (the largest).
+__host__ __device__ inline int64_t slice_red_size(int64_t N, int ncl) {
+  return tri_red_size((int)N / slice_count(N, ncl) + 1, kTriThreads);
 }
 // Factor storage of the preconditioner slices: slice (instance ii, rank) starts at
-// 5 (cell_off + c0 + (ii kCL + rank) kTriThreads), room for tri_fac_size(n, kTriThreads).
-__host__ __device__ inline int64_t prec_fac_off(int64_t cell_off, int64_t c0, int ii, int rank) {
-  return 5 * (cell_off + c0 + ((int64_t)ii * kCL + rank) * kTriThreads);
+// 5 (cell_off + c0 + (ii ncl + rank) kTriThreads), room for tri_fac_size(n, kTriThreads).
+__host__ __device__ inline int64_t prec_fac_off(int64_t cell_off, int64_t c0, int ii, int rank, int ncl) {
+  return 5 * (cell_off + c0 + ((int64_t)ii * ncl + rank) * kTriThreads);
 }
 
 struct GmresSmem {
@@ -678,7 +678,7 @@ struct GmresSmem {
   double xlr[2];                     // interface values left of and right of this slice
   double gfirst;                     // the moment G at the slice's first node (FP64)
   double y[kMaxRestart];
-  double prow[2][2 * kCL], pcol[2][2 * kCL];   // pivot row and column of the interface inversion
+  double prow[2][2 * kCLMax], pcol[2][2 * kCLMax];   // pivot row and column of the interface inversion
   double redm[kTriThreads / 32][kMaxRestart + 2];   // per-warp partials of a reduction
   double dots[2][kMaxRestart + 2];   // Gram-Schmidt coefficients of the two passes
   double cs[kMaxRestart], sn[kMaxRestart];     // Givens rotations of the earlier columns
@@ -714,6 +714,7 @@ __device__ double cta_sum(double v, double* red) {
 // Combine nv per-CTA values over the cluster in rank order: thread i < nv brings value i,
 // out[i] is the sum, from i = first_max on the maximum.  `buf` selects the half of the
 // double buffer; two consecutive calls must use different halves.
+template <int CL>
 __device__ __forceinline__ void cluster_combine(cg::cluster_group& cl, int na, GmresSmem& sm, int buf, double mine,
                                                 int nv, int first_max, double* out) {
   const int i = threadIdx.x;
@@ -721,12 +722,12 @@ __device__ __forceinline__ void cluster_combine(cg::cluster_group& cl, int na, G
     if (i < nv) sm.part[buf][i] = mine;
     cl.sync();
     if (i < nv) {
-      double v[kCL];
+      double v[CL];
 #pragma unroll
-      for (int r = 0; r < kCL; ++r) v[r] = r < na ? cl.map_shared_rank(&sm.part[buf][0], r)[i] : 0.0;
+      for (int r = 0; r < CL; ++r) v[r] = r < na ? cl.map_shared_rank(&sm.part[buf][0], r)[i] : 0.0;
       mine = v[0];
 #pragma unroll
-      for (int r = 1; r < kCL; ++r) mine = i >= first_max ? fmax(mine, v[r]) : mine + v[r];
+      for (int r = 1; r < CL; ++r) mine = i >= first_max ? fmax(mine, v[r]) : mine + v[r];
     }
   }
   if (i < nv) out[i] = mine;
@@ -739,7 +740,7 @@ __device__ __forceinline__ void cluster_combine(cg::cluster_group& cl, int na, G
 // Bound: latency (one CTA for up to 256 cells, eight above).  Eight basis vectors at a time, their
 // loads issued together; eight sums cross the warp in 4 + 2 + 1 + 1 + 1 shuffles instead
 // of 40.  Partial sums in K, reductions in double, in a fixed order.
-template <bool SQ, typename K>
+template <bool SQ, int CL, typename K>
 __device__ __forceinline__ void gs_dots(cg::cluster_group& cl, int na, GmresSmem& sm, int buf, const K* w,
                                         const K* V, int64_t ld, int64_t n, int nb, double* dots) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kTriThreads / 32;
@@ -786,7 +787,7 @@ __device__ __forceinline__ void gs_dots(cg::cluster_group& cl, int na, GmresSmem
   double t = 0.0;
   if (threadIdx.x < nv)
     for (int u = 0; u < nwa; ++u) t += sm.redm[u][threadIdx.x];
-  cluster_combine(cl, na, sm, buf, t, nv, nv, dots);
+  cluster_combine<CL>(cl, na, sm, buf, t, nv, nv, dots);
 }
 
 // z = P^{-1} r on this CTA's slice, P the single-effective-angle Schur operator:
@@ -797,7 +798,7 @@ __device__ __forceinline__ void gs_dots(cg::cluster_group& cl, int na, GmresSmem
 // coupling with the neighbouring slices); the 2*nact end values then give the
 // slice-boundary unknowns, and u = y - u_left g - u_right h.
 // K: arithmetic type of the Krylov vectors (the bulk type); RT: type of r.
-template <bool FACTOR, bool XS, typename K, typename RT>
+template <bool FACTOR, bool XS, int CL, typename K, typename RT>
 __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int rank, cg::cluster_group& cl,
                               const RT* r, K* z, K* work, K* wsm, GmresSmem& sm) {
   const int64_t N = I.N, co = I.cell_off, c0 = sl.c0, n = sl.n;
@@ -810,18 +811,19 @@ __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int 
   K* ph = (K*)D.pH + co;
   PrecCoef<K> pc{A, gl, gu, gb, ralpha, I.wv, I.wv2, N};
   SliceCoef<K> sc{pc, c0, n};
-  K* F = (K*)D.pF + prec_fac_off(co, c0, blockIdx.x / kCL, rank);
-  K* Rd = (K*)D.pRd + I.red_off + (int64_t)rank * (prec_red_size(N) / kCL);
+  K* F = (K*)D.pF + prec_fac_off(co, c0, blockIdx.x / CL, rank, CL);
+  K* Rd = (K*)D.pRd + I.red_off + (int64_t)rank * slice_red_size(N, CL);
   K* red = (K*)sm.tri;
   // the slice's unknowns: shared memory (XS) or the global work vector
   const XAcc<K, XS> wx{XS ? wsm : work + c0};
   const XAcc<K, false> gx{pg + c0}, hx{ph + c0};
   const int na = sl.nact, m2 = 2 * na;
-  double* inv_rows = D.pInv + ((int64_t)blockIdx.x) * 2 * (2 * kCL);
+  double* inv_rows = D.pInv + ((int64_t)blockIdx.x) * 2 * (2 * kCLMax);
   // the interface solve's coefficients (lane: side, column), loaded ahead of their use
-  const int iside = (threadIdx.x >> 4) & 1, icol = threadIdx.x & 15;
-  const bool ilive = threadIdx.x < 32 && icol < m2;
-  double iv = (!FACTOR && na > 1 && ilive) ? inv_rows[iside * 2 * kCL + icol] : 0.0;
+  constexpr int W = 2 * CL;   // columns of the interface matrix: 16 or 32
+  const int iside = threadIdx.x / W, icol = threadIdx.x % W;
+  const bool ilive = iside < 2 && icol < m2;
+  double iv = (!FACTOR && na > 1 && ilive) ? inv_rows[iside * 2 * kCLMax + icol] : 0.0;
   for (int64_t j = threadIdx.x; j < n; j += blockDim.x) wx[j] = ratio_k[c0 + j] * K(r[c0 + j]);
   __syncthreads();
   if (n > 0) {
@@ -851,39 +853,59 @@ __device__ void prec_apply_cl(const Dev& D, const Inst& I, const Slice& sl, int 
     //   X[2q+1] + g_last(q)  X[2q-1] + h_last(q)  X[2q+2] = y_last(q)
     // The matrix depends only on the operator: FACTOR inverts it once per step and stores
     // the two rows this slice needs; every apply is then two short dot products.  The
-    // inversion is in place, one element per thread, one barrier per pivot, without row
+    // inversion is in place, one or four elements per thread, one barrier per pivot, without row
     // exchanges: the spikes of a diagonally dominant system have |g| + |h| < 1 in every
     // row, so the matrix is diagonally dominant too.  (One warp with a pivot search and
     // the augmented matrix in shared memory took 30 us of a 128-cell step.)
     if (FACTOR) {
-      static_assert(kTriThreads == (2 * kCL) * (2 * kCL), "one thread per element of the interface matrix");
-      const int i = threadIdx.x / (2 * kCL), c = threadIdx.x % (2 * kCL);
-      double a = i == c ? 1.0 : 0.0;
-      if (i < m2) {
-        const int q = i / 2, t = i % 2;
-        const double* e = cl.map_shared_rank(&sm.ends[0], q);
-        if (q > 0 && c == 2 * q - 1) a += e[2 + t];
-        if (q < na - 1 && c == 2 * q + 2) a += e[4 + t];
+      // thread: column c of rows i0 + RS e
+      constexpr int RS = kTriThreads / W, E = W / RS;
+      const int i0 = threadIdx.x / W, c = threadIdx.x % W;
+      double a[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = i0 + RS * e;
+        a[e] = i == c ? 1.0 : 0.0;
+        if (i < m2) {
+          const int q = i / 2, t = i % 2;
+          const double* en = cl.map_shared_rank(&sm.ends[0], q);
+          if (q > 0 && c == 2 * q - 1) a[e] += en[2 + t];
+          if (q < na - 1 && c == 2 * q + 2) a[e] += en[4 + t];
+        }
       }
       for (int p = 0; p < m2; ++p) {
         const int b = p & 1;
-        if (i == p) sm.prow[b][c] = a;
-        if (c == p) sm.pcol[b][i] = a;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          if (i0 + RS * e == p) sm.prow[b][c] = a[e];
+          if (c == p) sm.pcol[b][i0 + RS * e] = a[e];
+        }
         __syncthreads();
-        const double ip = 1.0 / sm.prow[b][p];
-        const double rp = (c == p ? 1.0 : sm.prow[b][c]) * ip, f = sm.pcol[b][i];
-        a = i == p ? rp : (c == p ? -f * rp : a - f * rp);
+        const double ip = rcp64(sm.prow[b][p]);
+        const double rp = (c == p ? 1.0 : sm.prow[b][c]) * ip;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int i = i0 + RS * e;
+          if (i >= m2) continue;
+          const double f = sm.pcol[b][i];
+          a[e] = i == p ? rp : (c == p ? -f * rp : a[e] - f * rp);
+        }
       }
       // rows 2 rank - 1 and 2 rank + 2 of the inverse (zero at the ends of the grid)
       const bool hasL = rank > 0 && rank < na, hasR = rank < na - 1;
-      if (i == (hasL ? 2 * rank - 1 : 0)) inv_rows[c] = hasL ? a : 0.0;
-      if (i == (hasR ? 2 * rank + 2 : 0)) inv_rows[2 * kCL + c] = hasR ? a : 0.0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = i0 + RS * e;
+        if (i == (hasL ? 2 * rank - 1 : 0)) inv_rows[c] = hasL ? a[e] : 0.0;
+        if (i == (hasR ? 2 * rank + 2 : 0)) inv_rows[2 * kCLMax + c] = hasR ? a[e] : 0.0;
+      }
       __syncthreads();
-      if (ilive) iv = inv_rows[iside * 2 * kCL + icol];
+      if (ilive) iv = inv_rows[iside * 2 * kCLMax + icol];
     }
-    if (threadIdx.x < 32) {
+    if (threadIdx.x < (2 * W < 32 ? 32 : 2 * W)) {
       double acc = ilive ? iv * cl.map_shared_rank(&sm.ends[0], icol >> 1)[icol & 1] : 0.0;
-      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+#pragma unroll
+      for (int o = W / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (icol == 0) sm.xlr[iside] = acc;
     }
   } else if (threadIdx.x < 2) {
@@ -1050,8 +1072,8 @@ enum { G_RESTART_FIRST = 0, G_RESTART = 1, G_ARNOLDI = 2, G_UPDATE = 3 };
 // preconditioned).  Vectors live in global memory: x (iterate), V[0..m] (Krylov
 // basis), z (scratch).  Scalars (H, g, Givens) are computed identically by every
 // CTA; rank 0 stores them.
-template <int MODE, typename R, bool XS>
-__global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmres(Dev D, int jcol) {
+template <int MODE, typename R, bool XS, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kTriThreads) k_gmres(Dev D, int jcol) {
   using K = typename KryT<R>::type;   // arithmetic of the Krylov vectors
   // FP64 mode: the per-cell parts of the next pass are formed here (no separate launch)
   constexpr bool FUSED_PARTS = sizeof(R) == 8;
@@ -1060,10 +1082,10 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
   K* wsm = (K*)gdsm;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
-  const int ii = blockIdx.x / kCL;
+  const int ii = blockIdx.x / CL;
   const Inst I = D.inst[ii];
   const int64_t N = I.N, co = I.cell_off;
-  const Slice sl = slice_of(N, rank);
+  const Slice sl = slice_of<CL>(N, rank);
   const int64_t c0 = sl.c0, n = sl.n;
   const int m = D.m, na = sl.nact;
   if (na == 1 && rank > 0) return;   // a lone slice: no cluster barrier below
@@ -1110,8 +1132,8 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
     }
     __syncthreads();
     K* v0 = Vi(0);
-    if (MODE == G_RESTART_FIRST) prec_apply_cl<true, XS, K, double>(D, I, sl, rank, cl, r, v0, work, wsm, sm);
-    else prec_apply_cl<false, XS, K, double>(D, I, sl, rank, cl, r, v0, work, wsm, sm);
+    if (MODE == G_RESTART_FIRST) prec_apply_cl<true, XS, CL, K, double>(D, I, sl, rank, cl, r, v0, work, wsm, sm);
+    else prec_apply_cl<false, XS, CL, K, double>(D, I, sl, rank, cl, r, v0, work, wsm, sm);
     double xmax = 0.0;
     for (int q = 0; q < na; ++q)
       xmax = fmax(xmax, na > 1 ? cl.map_shared_rank(&sm.part[0][0], q)[0] : sm.part[0][0]);
@@ -1139,7 +1161,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
       for (int u = 0; u < nw; ++u)
         mine = threadIdx.x == 2 ? fmax(mine, sm.redm[u][2]) : mine + sm.redm[u][threadIdx.x];
     double* tots = sm.dots[0];   // |v|^2, |x|^2, the largest weighted |v_j|
-    cluster_combine(cl, na, sm, 1, mine, 3, 2, tots);
+    cluster_combine<CL>(cl, na, sm, 1, mine, 3, 2, tots);
     const double nrm = sqrt(tots[0]), xn = sqrt(tots[1]);
     const double rinf = tots[2];
     // Converged when every cell's relative preconditioned correction is below rtol.
@@ -1200,7 +1222,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
       cv[j] = alpha_k[j] * vj[j] + kdx_k[j] * K(flux_sum_k<R>(D, I, j, G));
     __syncthreads();
     K* wv = Vi(jcol + 1);
-    prec_apply_cl<false, XS, K, K>(D, I, sl, rank, cl, cv, wv, work, wsm, sm);
+    prec_apply_cl<false, XS, CL, K, K>(D, I, sl, rank, cl, cv, wv, work, wsm, sm);
     // classical Gram-Schmidt, twice (CGS2), w in shared memory (XS): each thread works on
     // its own cells only.  The second pass's reduction also carries |w|^2, from which the
     // norm after it is |w|^2 - sum_i d_i^2 (its coefficients d_i are rounding-level, so
@@ -1209,7 +1231,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
     K* w = XS ? wsm : wv + c0;
     if (XS)
       for (int64_t j = threadIdx.x; j < n; j += blockDim.x) w[j] = wv[c0 + j];
-    gs_dots<false>(cl, na, sm, 0, w, V + c0, ncell_tot, n, nb, sm.dots[0]);
+    gs_dots<false, CL>(cl, na, sm, 0, w, V + c0, ncell_tot, n, nb, sm.dots[0]);
     auto gs_sub = [&](const double* d, double scale, K* out) {
       for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
         K t = w[j];
@@ -1225,7 +1247,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kTriThreads) k_gmr
       }
     };
     gs_sub(sm.dots[0], 1.0, w);
-    gs_dots<true>(cl, na, sm, 1, w, V + c0, ncell_tot, n, nb, sm.dots[1]);
+    gs_dots<true, CL>(cl, na, sm, 1, w, V + c0, ncell_tot, n, nb, sm.dots[1]);
     double nn = sm.dots[1][nb];
     for (int i = 0; i < nb; ++i) nn -= sm.dots[1][i] * sm.dots[1][i];
     const double inrm = nn > 0.0 ? rsqrt(nn) : 0.0;
@@ -1715,13 +1737,16 @@ static cudaError_t line_kernel_attrs() {
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, f);
     if (e == cudaSuccess) gdyn = std::min(gdyn, bytes - (int)fa.sharedSizeBytes);
   };
-  const void* gk[] = {(const void*)k_gmres<G_RESTART_FIRST, double, true>, (const void*)k_gmres<G_RESTART, double, true>,
-                      (const void*)k_gmres<G_ARNOLDI, double, true>, (const void*)k_gmres<G_UPDATE, double, true>,
-                      (const void*)k_gmres<G_RESTART_FIRST, float, true>, (const void*)k_gmres<G_RESTART, float, true>,
-                      (const void*)k_gmres<G_ARNOLDI, float, true>, (const void*)k_gmres<G_UPDATE, float, true>};
+#define GK(R, XS, CL) (const void*)k_gmres<G_RESTART_FIRST, R, XS, CL>, (const void*)k_gmres<G_RESTART, R, XS, CL>, \
+                      (const void*)k_gmres<G_ARNOLDI, R, XS, CL>, (const void*)k_gmres<G_UPDATE, R, XS, CL>
+  const void* gk[] = {GK(double, true, kCL), GK(float, true, kCL), GK(double, true, kCLMax)};
+  const void* wide[] = {GK(double, true, kCLMax), GK(double, false, kCLMax)};
+#undef GK
   for (const void* f : gk) gm(f);
   for (const void* f : gk)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, gdyn);
+  for (const void* f : wide)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   g_gmres_dyn = gdyn;
   if (dev >= 0 && dev < 64) done[dev] = true;
@@ -1731,11 +1756,35 @@ static cudaError_t line_kernel_attrs() {
 static int64_t gmres_dyn_smem(const grte_ctx* h) {
   return h->gxs ? (tri_xs_len(h->max_slice) * 8 + 15) / 16 * 16 : 0;
 }
+template <int MODE, typename R, int CL>
+static void gmres_launch_cl(grte_ctx* h, int jcol) {
+  const unsigned grid = (unsigned)(h->n_inst * CL);
+  if (h->gxs) k_gmres<MODE, R, true, CL><<<grid, kTriThreads, (size_t)gmres_dyn_smem(h), h->stream>>>(h->D, jcol);
+  else k_gmres<MODE, R, false, CL><<<grid, kTriThreads, 0, h->stream>>>(h->D, jcol);
+}
 template <int MODE, typename R>
 static void gmres_launch(grte_ctx* h, int jcol) {
-  const unsigned grid = (unsigned)(h->n_inst * kCL);
-  if (h->gxs) k_gmres<MODE, R, true><<<grid, kTriThreads, (size_t)gmres_dyn_smem(h), h->stream>>>(h->D, jcol);
-  else k_gmres<MODE, R, false><<<grid, kTriThreads, 0, h->stream>>>(h->D, jcol);
+  if constexpr (sizeof(R) == 8)
+    if (h->D.ncl == kCLMax) return gmres_launch_cl<MODE, R, kCLMax>(h, jcol);
+  gmres_launch_cl<MODE, R, kCL>(h, jcol);
+}
+
+// Cluster size of the Krylov kernels.  Sixteen CTAs halve the binary64 work per SM, which
+// bounds a large FP64 instance: us per kernel with 8 / 16 CTAs, 32 angles, 55.9 / 43.9 at 8192
+// cells, 40.3 / 33.4 at 4096, 29.7 / 28.8 at 2048, 28.8 / 30.6 at 1500, 26.6 / 28.7 at 1000.  But
+// they fill a GPC, so seven such clusters fit at a time: 12 runs of 2048 cells take 29.4 / 30.5.
+constexpr int64_t kWideCells = 2048;
+constexpr int kWideInst = 7;
+static int gmres_cluster(int n_inst, int64_t max_nx, bool mixed) {
+  if (mixed || n_inst > kWideInst || max_nx < kWideCells) return kCL;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCLMax);
+  cfg.blockDim = dim3(kTriThreads);
+  int n = 0;
+  const cudaError_t e =
+      cudaOccupancyMaxActiveClusters(&n, (const void*)k_gmres<G_RESTART_FIRST, double, true, kCLMax>, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess && n >= 1 ? kCLMax : kCL;
 }
 
 template <int MODE, typename R, int NT, bool XS>
@@ -1998,7 +2047,7 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   if (h->opt.krylov_restart < 1 || h->opt.krylov_restart > kMaxRestart) return bad("krylov_restart out of range [1,16]");
   if (h->opt.krylov_maxcycles < 1 || h->opt.newton_maxit < 1 || !(h->opt.krylov_rtol > 0)) return bad("bad solver options");
   h->n_inst = n_inst;
-  int64_t coff = 0, eoff = 0, noff = 0, roff = 0, poff = 0, foff = 0;
+  int64_t coff = 0, eoff = 0, noff = 0, roff = 0, foff = 0;
   int aoff = 0, loff = 0;
   if (h->opt.line_threads != 0 && h->opt.line_threads != 256 && h->opt.line_threads != 512 &&
       h->opt.line_threads != 1024)
@@ -2065,7 +2114,6 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
     I.cell_off = coff;
     I.elem_off = eoff;
     I.nelem_off = noff;
-    I.red_off = poff;
     I.ang_off = aoff;
     I.line_off = loff;
     for (int k = 0; k < p.n_angle; ++k) {
@@ -2074,10 +2122,6 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
       foff += 5 * (p.nx + std::min<int64_t>(p.nx / 2, kTriMaxNT));   // >= tri_fac_size(nx, nt), nt <= 1024
     }
     h->maxN = std::max<int64_t>(h->maxN, p.nx);
-    {
-      h->max_slice = std::max<int64_t>(h->max_slice, p.nx / slice_count(p.nx) + 1);
-    }
-    poff += prec_red_size(p.nx);
     coff += p.nx;
     eoff += p.nx * p.n_angle;
     noff += (p.nx + 1) * p.n_angle;
@@ -2092,7 +2136,6 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   h->nelem = eoff;
   h->nnelem = noff;
   h->nred = roff;
-  h->npred = poff;
   *out = h;
   if (h->opt.stream) {
     h->stream = (cudaStream_t)h->opt.stream;
@@ -2102,6 +2145,13 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   }
   CK(cudaEventCreateWithFlags(&h->ev_state, cudaEventDisableTiming));
   Dev& D = h->D;
+  CK(line_kernel_attrs());
+  D.ncl = gmres_cluster(n_inst, h->maxN, h->opt.precision == GRTE_MIXED);
+  for (Inst& I : h->inst) {
+    h->max_slice = std::max<int64_t>(h->max_slice, I.N / slice_count(I.N, D.ncl) + 1);
+    I.red_off = h->npred;
+    h->npred += D.ncl * slice_red_size(I.N, D.ncl);
+  }
   const int m = h->opt.krylov_restart;
   D.m = m;
   D.maxcycles = h->opt.krylov_maxcycles;
@@ -2152,8 +2202,8 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
     if (dalloc(h, &p_, es * h->nred) != cudaSuccess) return nomem("cudaMalloc Rd"); D.Rd = p_;
     if (dalloc(h, &p_, es * nn) != cudaSuccess) return nomem("cudaMalloc onode"); D.onode = p_;
   }
-  AL(D.pF, 5 * (nc + (int64_t)n_inst * kCL * kTriThreads)); AL(D.pRd, h->npred); AL(D.pG, nc); AL(D.pH, nc);
-  AL(D.pInv, (int64_t)n_inst * kCL * 2 * (2 * kCL));
+  AL(D.pF, 5 * (nc + (int64_t)n_inst * D.ncl * kTriThreads)); AL(D.pRd, h->npred); AL(D.pG, nc); AL(D.pH, nc);
+  AL(D.pInv, (int64_t)n_inst * D.ncl * 2 * (2 * kCLMax));
   // x, z contiguous so that the GMRES kernel can recover the total cell count
   double* xz = nullptr;
   AL(xz, 2 * nc);
@@ -2199,7 +2249,6 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   CK(cudaMemcpy(D.sig, hsig.data(), sizeof(double) * nc, cudaMemcpyHostToDevice));
   CK(cudaMallocHost(&h->h_flags, sizeof(int) * n_inst));
   h->inst_set.assign(n_inst, 0);
-  CK(line_kernel_attrs());
   // line solves: unknowns in shared memory when the largest line fits at 256 threads
   h->xs = line_fits(h, 256);
   h->gxs = (tri_xs_len(h->max_slice) * 8 + 15) / 16 * 16 <= g_gmres_dyn;
@@ -3192,15 +3241,15 @@ constexpr int64_t kNaBytes =
     na_round(8 * kNaMaxNodeElems) +                                 // node scratch
     na_round(8 * kNaMaxAngles * kNaRedLine) +                        // line reduced systems
     na_round(8 * 5 * kNaMaxAngles) + na_round(8 * 2 * kNaMaxAngles) +   // v, w, bL, bR, w v^2; Swall
-    na_round(8 * ((kMaxRestart + 1) * kMaxRestart + 3 * kMaxRestart + 8 + kCL * 2 * 2 * kCL)) +
+    na_round(8 * ((kMaxRestart + 1) * kMaxRestart + 3 * kMaxRestart + 8 + kCL * 2 * 2 * kCLMax)) +
     na_round(4 * 16) + na_round(sizeof(Inst)) + na_round(sizeof(Line) * kNaMaxAngles) + na_round(8);
 }  // namespace grte
 
-// Work memory of grte_step1d_noalloc: kNaBytes = 10,707,200 bytes (about 10.7 MB),
+// Work memory of grte_step1d_noalloc: kNaBytes = 10,709,248 bytes (about 10.7 MB),
 // held by every GPU that loads the library until the process exits.  Calls share it
 // (see include/grte.h, which states the same figure; the assertion keeps the two in
 // step when the layout changes).
-static_assert(grte::kNaBytes == 10707200, "no-alloc work memory size changed: update the documented figure");
+static_assert(grte::kNaBytes == 10709248, "no-alloc work memory size changed: update the documented figure");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[grte::kNaBytes];
 static void* g_noalloc_base[64];   // device address of g_noalloc_scratch, per device
 
@@ -3344,7 +3393,7 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
   double* vw = (double*)take(8 * 5 * kNaMaxAngles);
   D.v = vw; D.w = vw + kNaMaxAngles; D.bL = vw + 2 * kNaMaxAngles; D.bR = vw + 3 * kNaMaxAngles; D.wvv = vw + 4 * kNaMaxAngles;
   D.Swall = (double*)take(8 * 2 * kNaMaxAngles);
-  double* small = (double*)take(8 * ((kMaxRestart + 1) * kMaxRestart + 3 * kMaxRestart + 8 + kCL * 2 * 2 * kCL));
+  double* small = (double*)take(8 * ((kMaxRestart + 1) * kMaxRestart + 3 * kMaxRestart + 8 + kCL * 2 * 2 * kCLMax));
   D.gH = small;
   D.gg = D.gH + (kMaxRestart + 1) * kMaxRestart;
   D.gcs = D.gg + kMaxRestart + 1;
@@ -3361,6 +3410,7 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
   int64_t* d_cell_start = (int64_t*)take(8);
   if (cur - (unsigned char*)g_noalloc_base[dev] > kNaBytes) return GRTE_ENOMEM;   // layout check
   D.T = T;
+  D.ncl = kCL;
   D.O = O;
   D.inst = d_inst;
   D.lines = d_lines;
@@ -3387,7 +3437,7 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
   NA(cudaMemcpyAsync(D.sig, p->sigma, 8 * N, cudaMemcpyHostToDevice, st));
   // what must start at zero: statuses, counters, energy sums, Krylov scalars
   NA(cudaMemsetAsync(ints, 0, 4 * 16, st));
-  NA(cudaMemsetAsync(small, 0, 8 * ((kMaxRestart + 1) * kMaxRestart + 3 * kMaxRestart + 8 + kCL * 2 * 2 * kCL), st));
+  NA(cudaMemsetAsync(small, 0, 8 * ((kMaxRestart + 1) * kMaxRestart + 3 * kMaxRestart + 8 + kCL * 2 * 2 * kCLMax), st));
   const double ac = p->a * p->c;
   const unsigned eb = (unsigned)((N * M + 255) / 256);
   k_na_prepare<<<eb, 256, 0, st>>>(T, E, D.U, (double*)D.Eh, N, M, ac);
@@ -3413,7 +3463,7 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
   if (line_kernel_attrs() != cudaSuccess) { ctx.h_flags = nullptr; return GRTE_ECUDA; }
   ctx.maxN = N;
   ctx.xs = line_fits(&ctx, kTriThreads);
-  ctx.max_slice = N / slice_count(N) + 1;
+  ctx.max_slice = N / slice_count(N, kCL) + 1;
   ctx.gxs = (tri_xs_len(ctx.max_slice) * 8 + 15) / 16 * 16 <= g_gmres_dyn;
   ctx.nt = kTriThreads;
   for (int64_t n = 0; n < nsteps; ++n) {
