@@ -147,3 +147,23 @@ def test_2d_restart_lengths(G, restart):
         res.append(h.T(allow=(5,)))
         h.close()
     assert np.max(np.abs(res[1] - res[0]) / res[0]) < 1e-9
+
+
+# The gradient of n samples is the mean of those of its parts (block edges at 64, eight groups of
+# blocks in the reduction).  The same products in both: only binary32 sums of up to n terms are
+# ordered differently, 1e-5 of the largest entry; the samples' BF16 operands are the same but for
+# the 1/n in front, which moves their rounding by up to 2^-8 of single terms: 2e-3.
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 448, 512, 513, 577])
+def test_gradient_block_edges(G, n):
+    rng = np.random.default_rng(12)
+    m = G.MLP(seed=4)
+    m.set_norm(np.zeros(6, np.float32), np.ones(6, np.float32), 0.0, 1.0)
+    X = rng.standard_normal((n, 6)).astype(np.float32)
+    Y = rng.standard_normal(n).astype(np.float32)
+    loss, g = m.grad(X, Y)
+    parts = [(len(X[i:i + 50]), m.grad(X[i:i + 50], Y[i:i + 50])) for i in range(0, n, 50)]
+    want_l = sum(k * p[0] for k, p in parts) / n
+    want = sum(k * p[1].astype(np.float64) for k, p in parts) / n
+    assert abs(loss - want_l) < 1e-5 * want_l
+    assert np.max(np.abs(g - want)) < 2e-3 * np.max(np.abs(want))
+    m.close()
