@@ -1407,7 +1407,7 @@ static grte_status step2(grte2d_t h) {
   // prediction's coefficients (sigma(x)) or those of V* = (U*)^{3/4} (sigma_0/T^3)
   if (g.kind == GRTE_SIGMA_T3) {
     // the prediction's vertex values (the Krylov basis is free until the correction's
-    // solve: it holds (m+1)(K+1) nc >= K nv values), then those of V*; the inflow walls
+    // solve and has room for K nv values), then those of V*; the inflow walls
     // shifted (k2_wallshift) and the wall-normal parts of the wall cells taken from the
     // prediction's (k2_fdiv_corr)
     double* Vp = h->Kbasis;
@@ -1551,7 +1551,9 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
             alloc2(h, &D.wsc, nc) && alloc2(h, &D.iwsc, nc) && alloc2(h, &D.gd, K * nc) && alloc2(h, &D.gdi, K * nc) && alloc2(h, &D.pdi, nc) &&
             alloc2(h, &h->V, K * nv) && alloc2(h, &h->phi, K * nc) && alloc2(h, &h->GU, K * nc) &&
             alloc2(h, &h->Es, K * nc) && alloc2(h, &h->b, nz) && alloc2(h, &h->x, nz) && alloc2(h, &h->Kr, nz) &&
-            alloc2(h, &h->Kt, nz) && alloc2(h, &h->Kbasis, (int64_t)(h->m + 1) * basis_ld(nz)) &&
+            alloc2(h, &h->Kt, nz) &&
+            // also the scratch of K nv vertex values between solves (2 x 2 cells, m = 1: the larger)
+            alloc2(h, &h->Kbasis, std::max((int64_t)(h->m + 1) * basis_ld(nz), K * nv)) &&
             alloc2(h, &h->part, (int64_t)kAxpyBlocks * (kMaxRestart2 + 1)) && alloc2(h, &h->dots, kMaxRestart2 + 1) &&
             alloc2(h, &h->cscale, nc) && alloc2(h, &h->tk, K * nc) && alloc2(h, &h->ks, 1) && alloc2(h, &h->count, 1);
   if (!ok) return fail2(h, GRTE_ENOMEM, "cudaMalloc failed");
