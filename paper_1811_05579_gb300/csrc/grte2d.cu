@@ -35,6 +35,7 @@ struct NvtxRange {
 #include "mg2d.cuh"
 #include "mgpair2d.cuh"
 #include "mlp.cuh"
+#include "rows2d.h"
 #include "stateio.cuh"
 
 namespace grte2 {
@@ -1485,7 +1486,7 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
   if (!(h->opt.krylov_rtol > 0) || h->opt.krylov_maxcycles < 1 || h->opt.newton_maxit < 1)
     return fail2(h, GRTE_EINVAL, "bad solver options");
   if (p->nx < 2 || p->ny < 2 || p->nx > 32768 || p->ny > 32768) return fail2(h, GRTE_EINVAL, "nx, ny must be in [2, 32768]");
-  if ((int64_t)std::max(p->n_pair, 20) * (p->nx + 1) * (p->ny + 1) >= (int64_t)1 << 31)
+  if (!rows_fit(p->n_pair, p->nx, p->ny))
     return fail2(h, GRTE_EINVAL, "n_pair * (nx+1) * (ny+1) must be below 2^31");
   if (!p->sigma) return fail2(h, GRTE_EINVAL, "sigma is NULL");
   if (p->sigma_kind != GRTE_SIGMA_CONST && p->sigma_kind != GRTE_SIGMA_T3 && p->sigma_kind != GRTE_SIGMA_POW)

@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(TX * TY * G, op_min_blocks<S, TX, TY, G>())
   static_assert(NH <= NT && NE <= NT, "one halo cell and one edge vertex per thread");
   extern __shared__ __align__(16) unsigned char op_raw[];
   const G2& g = D.g;
-  const int K = g.K, nc = (int)g.nc;                // K nc < 2^31 (checked at creation)
+  const int K = g.K, nc = (int)g.nc;                // K nc < 2^31 (rows_fit) but not (K+1) nc:
+  const int64_t rrow = rho_row(K, nc);              // the rho row's indices have 64 bits
   const int tid = threadIdx.x % NT, gq = threadIdx.x / NT, lx = tid % TX, ly = tid / TX;
   S* p = reinterpret_cast<S*>(op_raw);
   S* const tu = p + gq * NC;   p += G * NC;         // u of the group's pair
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(TX * TY * G, op_min_blocks<S, TX, TY, G>())
   // (past the domain: a halo cell of a live one, or on a periodic axis its image)
   const int c = live ? qc * g.Nx + pc : cell_of(g, pc, qc);
   const S fc = c >= 0 ? (sc ? sc[c] * iv : iv) : S(0);
-  const S rc = PRED && c >= 0 ? z[K * nc + c] * fc : S(0);
+  const S rc = PRED && c >= 0 ? z[rrow + c] * fc : S(0);
   const S A = live ? cv.A[c] : S(0), kc = live ? cv.kc[c] : S(0), al = PRED && live ? cv.alpha[c] : S(0);
   const S ws = PREC && live ? cv.wsc[c] : S(1), arc = al * rc;
   const bool xw = g.bcx == GRTE_BC_INFLOW, yw = g.bcy == GRTE_BC_INFLOW;
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(TX * TY * G, op_min_blocks<S, TX, TY, G>())
     hc = cell_of(g, p0 - 1 + hx, q0 - 1 + hy);
     if (hc >= 0) {
       hf = sc ? sc[hc] * iv : iv;
-      if (PRED) hu = z[K * nc + hc] * hf;
+      if (PRED) hu = z[rrow + hc] * hf;
     }
   }
   // its vertices: the cell's lower left one, and one of the upper row or right column
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(TX * TY * G, op_min_blocks<S, TX, TY, G>())
     }
   }
   if (!live) return;
-  const int orho = K * nc + c;
+  const int64_t orho = rrow + c;
   S rr = fma(al, rc, st);
   if (RES) rr = b[orho] - rr;
   if (!PREC) {
