@@ -624,7 +624,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_pred_line(Dev D, const void* 
 // distributed shared memory (fixed rank order, so every CTA gets the same value);
 // the preconditioner's tridiagonal solve is partitioned across the cluster by the
 // spike method (local solves plus a 2 ncl interface system).
-constexpr int kCL = 8, kCLMax = 16;
 
 template <typename K>
 struct PrecCoef {  // A + (A/alpha) (wv2 Gint + wv Gbdry), evaluated in double, stored in K
@@ -651,14 +650,6 @@ struct Slice {
   int64_t c0, n;   // this CTA's cells [c0, c0+n) (n = 0 if rank >= nact)
 };
 
-// CTAs that share the N cells of one instance: a lone one up to a cell per thread, above
-// that the whole cluster.  The work on a slice is a chain of short dependent steps, so a
-// CTA takes hardly longer for 128 cells than for 16, and a lone slice needs no cluster
-// barrier, no spikes and no interface system: all Krylov kernels of a 128-cell step took
-// 190 us over 8 slices, 184 over 2 and 165 in one; at 1000 cells 132 us over 8 slices
-// and 137 over 4.
-constexpr int kLoneCells = kTriThreads;
-__host__ __device__ inline int slice_count(int64_t N, int ncl) { return N <= kLoneCells ? 1 : ncl; }
 template <int CL>
 __device__ __forceinline__ Slice slice_of(int64_t N, int rank) {
   Slice sl;
@@ -1763,7 +1754,7 @@ static cudaError_t line_kernel_attrs() {
 }
 
 static int64_t gmres_dyn_smem(const grte_ctx* h) {
-  return h->gxs ? (tri_xs_len(h->max_slice) * 8 + 15) / 16 * 16 : 0;
+  return gmres_dyn_bytes(h->max_slice, g_gmres_dyn);
 }
 template <int MODE, typename R, int CL>
 static void gmres_launch_cl(grte_ctx* h, int jcol) {
@@ -1778,23 +1769,27 @@ static void gmres_launch(grte_ctx* h, int jcol) {
   gmres_launch_cl<MODE, R, kCL>(h, jcol);
 }
 
-// Cluster size of the Krylov kernels.  Sixteen CTAs halve the binary64 work per SM, which
-// bounds a large FP64 instance: us per kernel with 8 / 16 CTAs, 32 angles, 55.9 / 43.9 at 8192
-// cells, 40.3 / 33.4 at 4096, 29.7 / 28.8 at 2048, 28.8 / 30.6 at 1500, 26.6 / 28.7 at 1000.  But
-// they fill a GPC, so seven such clusters fit at a time: 12 runs of 2048 cells take 29.4 / 30.5.
-constexpr int64_t kWideCells = 2048;
-constexpr int kWideInst = 7;
-static int gmres_cluster(int n_inst, int64_t max_nx, bool mixed) {
-  if (mixed || n_inst > kWideInst || max_nx < kWideCells) return kCL;
+// Whether a cluster of sixteen CTAs of the FP64 Krylov kernels with dyn bytes of dynamic shared
+// memory each (0: the unknowns in global memory) can be resident, the launches' configuration.
+template <bool XS>
+static bool wide_resident_xs(int64_t dyn) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCLMax);
   cfg.blockDim = dim3(kTriThreads);
-  int n = 0;
-  const cudaError_t e =
-      cudaOccupancyMaxActiveClusters(&n, (const void*)k_gmres<G_RESTART_FIRST, double, true, kCLMax>, &cfg);
-  if (e != cudaSuccess) cudaGetLastError();
-  return e == cudaSuccess && n >= 1 ? kCLMax : kCL;
+  cfg.dynamicSmemBytes = (size_t)dyn;
+  const void* k[] = {(const void*)k_gmres<G_RESTART_FIRST, double, XS, kCLMax>, (const void*)k_gmres<G_RESTART, double, XS, kCLMax>,
+                     (const void*)k_gmres<G_ARNOLDI, double, XS, kCLMax>, (const void*)k_gmres<G_UPDATE, double, XS, kCLMax>};
+  for (const void* f : k) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (n < 1) return false;
+  }
+  return true;
 }
+static bool wide_resident(int64_t dyn) { return dyn > 0 ? wide_resident_xs<true>(dyn) : wide_resident_xs<false>(0); }
 
 template <int MODE, typename R, int NT, bool XS>
 static void pred_launch(grte_ctx* h, const void* x) {
@@ -2155,9 +2150,11 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   CK(cudaEventCreateWithFlags(&h->ev_state, cudaEventDisableTiming));
   Dev& D = h->D;
   CK(line_kernel_attrs());
-  D.ncl = gmres_cluster(n_inst, h->maxN, h->opt.precision == GRTE_MIXED);
+  std::vector<int64_t> sizes;
+  for (const Inst& I : h->inst) sizes.push_back(I.N);
+  D.ncl = gmres_cluster(sizes.data(), n_inst, h->opt.precision == GRTE_MIXED, g_gmres_dyn, wide_resident);
+  h->max_slice = largest_slice(sizes.data(), n_inst, D.ncl);
   for (Inst& I : h->inst) {
-    h->max_slice = std::max<int64_t>(h->max_slice, I.N / slice_count(I.N, D.ncl) + 1);
     I.red_off = h->npred;
     h->npred += D.ncl * slice_red_size(I.N, D.ncl);
   }
@@ -2260,7 +2257,7 @@ grte_status grte_create_1d(int n_inst, const grte_instance1d* in, const grte_opt
   h->inst_set.assign(n_inst, 0);
   // line solves: unknowns in shared memory when the largest line fits at 256 threads
   h->xs = line_fits(h, 256);
-  h->gxs = (tri_xs_len(h->max_slice) * 8 + 15) / 16 * 16 <= g_gmres_dyn;
+  h->gxs = gmres_dyn_bytes(h->max_slice, g_gmres_dyn) > 0;
   if (h->opt.line_threads != 0) h->nt = (h->xs && line_fits(h, h->opt.line_threads)) ? h->opt.line_threads : 256;
   else if (!h->xs) h->nt = 256;   // nothing to tune: the global-memory variant runs at 256
   // fused prediction solve: mixed precision, every instance within the slice limits, and a
@@ -3467,8 +3464,8 @@ extern "C" grte_status grte_step1d_noalloc(const grte_instance1d* p, const grte_
   if (line_kernel_attrs() != cudaSuccess) { ctx.h_flags = nullptr; return GRTE_ECUDA; }
   ctx.maxN = N;
   ctx.xs = line_fits(&ctx, kTriThreads);
-  ctx.max_slice = N / slice_count(N, kCL) + 1;
-  ctx.gxs = (tri_xs_len(ctx.max_slice) * 8 + 15) / 16 * 16 <= g_gmres_dyn;
+  ctx.max_slice = largest_slice(&N, 1, kCL);
+  ctx.gxs = gmres_dyn_bytes(ctx.max_slice, g_gmres_dyn) > 0;
   ctx.nt = kTriThreads;
   for (int64_t n = 0; n < nsteps; ++n) {
     grte_status s = step_once<double>(&ctx);

@@ -23,9 +23,10 @@
 #pragma once
 #include <cstdint>
 
+#include "gmres_rule.h"
+
 namespace grte {
 
-constexpr int kTriThreads = 256;          // threads per CTA of the preconditioner slices
 constexpr int kTriMaxNT = 1024;           // largest thread count of a line CTA
 constexpr int kMaxLevels = 11;            // PCR levels for up to 2*kTriMaxNT reduced equations
 constexpr int kB = 8;                     // elements per block of the serial sweeps
@@ -55,8 +56,6 @@ __host__ __device__ inline int64_t tri_fac_size(int64_t n, int nt) { return 5 * 
 __host__ __device__ inline int64_t tri_smem_bytes(int nt, bool factor, int elem) {
   return (int64_t)(factor ? 4 : 2) * 2 * nt * elem;
 }
-// padded length of a shared-memory x of n values
-__host__ __device__ inline int64_t tri_xs_len(int64_t n) { return n + (n >> 5) + 1; }
 
 template <typename R, bool SM>
 struct XAcc {
