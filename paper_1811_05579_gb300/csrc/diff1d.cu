@@ -239,6 +239,12 @@ __device__ __forceinline__ void d_eliminate(const double* a, const double* b, co
   R = fma(-a[3], k.rc[2], r[3]);
 }
 
+// The power of two s with 1 <= den s < 2 (den > 0; at the ends of the range the nearest one).
+__device__ __forceinline__ double d_inv_scale(double den) {
+  const int e = __double2hiint(den) & 0x7ff00000;
+  return __hiloint2double(max(0x7fe00000 - e, 0x00100000), 0);
+}
+
 // Parallel cyclic reduction over lanes [0, n) of a warp, rows with unit diagonal:
 // x_i + a x_{i-1} + c x_{i+1} = r.  A coupling beyond either end is kept: afterwards
 // x_i = r - a x_{-1} - c x_n.
@@ -268,8 +274,9 @@ __device__ __forceinline__ void d_pcr(int lane, int n, double& a, double& c, dou
 
 // nsteps steps of one instance per cluster of Q = ceil(N/512) CTAs: CTA q holds cells
 // [512 q, 512 q + 512), four consecutive ones per thread, T and the node factors in registers.
-// Stage 1 multiplied by dt (a T^3 + C_v/4) needs no division per cell:
-//   [den + T^3 (k_j + k_{j+1})] U*_j - T^3 (k_j U*_{j-1} + k_{j+1} U*_{j+1}) = den U_j.
+// Stage 1 multiplied by dt (a T^3 + C_v/4) = dt den needs no division per cell:
+//   [den + T^3 (k_j + k_{j+1})] U*_j - T^3 (k_j U*_{j-1} + k_{j+1} U*_{j+1}) = den U_j,
+// each row scaled by a power of two so that den U_j ~ T^7 cannot leave the range before U_j does.
 // Four levels of elimination, the last unknown of each group kept as its separator: 4 cells
 // per thread; 4 threads' separators per lane of warp 0; 31 lanes by cyclic reduction with the
 // couplings to both ends carried along; one row per CTA, gathered by every CTA's warp 0.
@@ -331,11 +338,13 @@ __global__ void __launch_bounds__(kFT) k_diff(DDev D, int first, int Q, int nste
       double a[kFC], b[kFC], c[kFC], r[kFC];
 #pragma unroll
       for (int u = 0; u < kFC; ++u) {
-        const double den = fma(I.a, T3[u], c4);
-        a[u] = -T3[u] * kn[u];
-        c[u] = -T3[u] * kn[u + 1];
-        b[u] = den - (a[u] + c[u]);
-        r[u] = den * U[u];
+        // the row times a power of two that brings den to [1, 2): exact, and den U* stays in range
+        // wherever U* does
+        const double den = fma(I.a, T3[u], c4), s = d_inv_scale(den), T3s = T3[u] * s, dens = den * s;
+        a[u] = -T3s * kn[u];
+        c[u] = -T3s * kn[u + 1];
+        b[u] = dens - (a[u] + c[u]);
+        r[u] = dens * U[u];
       }
       d_eliminate(a, b, c, r, k, A, B, R);
       cx = c[kFC - 1];
