@@ -103,7 +103,7 @@ __device__ __forceinline__ bool d_root(double beta, double R, int maxit, double&
 __device__ __forceinline__ double d_correct(double beta, double R, int maxit, int& status) {
   double t = 0.0;
   if (!(R > 0.0)) {
-    if (R <= 0.0) status |= 1 << GRTE_ENEGATIVE;
+    status |= 1 << (R <= 0.0 ? GRTE_ENEGATIVE : GRTE_ENAN);
   } else if (!d_root(beta, R, maxit, t)) {
     status |= 1 << GRTE_ENONCONV;
   }
