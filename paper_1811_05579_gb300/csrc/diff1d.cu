@@ -307,7 +307,8 @@ __global__ void __launch_bounds__(kFT) k_diff(DDev D, int first, int Q, int nste
     g[u] = 0.0;
     if (i >= 1 && i < I.N) {
       const double sl = D.sig[I.off + i - 1], sr = D.sig[I.off + i];
-      g[u] = I.dt * I.a * I.c * (sl + sr) / (I.Dd * 2.0 * sl * sr * I.dx * I.dx) * (t3k ? 0.5 : 1.0);
+      const double sn = 2.0 * sl * sr / (sl + sr);   // (as k_dcoef: no product of more than two sigma)
+      g[u] = I.dt * (I.a * I.c / (I.Dd * sn * I.dx * I.dx)) * (t3k ? 0.5 : 1.0);
     }
   }
   int status = 0;

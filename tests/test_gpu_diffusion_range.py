@@ -69,3 +69,21 @@ def test_far_from_one(G, unit, exps):
 # (three launches solve for U*/dt rows, which leave the range earlier)
 def test_up_to_the_end_of_the_range(G, unit):
     check(G, unit, dict(const=250), sizes=(100, 700))
+
+
+# sigma -> s sigma, dt -> s dt leaves a step as it is: the node factor's sigma_l sigma_r stays in the
+# binary64 range at s = 2^-510 (sigma >= 1), times dx^2 it would have 28 bits left.
+def test_small_sigma(G):
+    rng = np.random.default_rng(98)
+    N, s = 8192, 2.0 ** -510
+    x = (np.arange(N) + 0.5) / N
+    T0, sig, dt = 1.0 + 0.4 * np.sin(2 * np.pi * x), 1.0 + rng.random(N), 0.05 / N
+    for kind, okind in ((G.SIGMA_CONST, "const"), (G.SIGMA_T3, "t3")):
+        T, Us = dif.three_stage_step(T0, sig, 1.0 / N, dt, kind=okind)
+        h = G.Diffusion([dict(nx=N, sigma=sig * s, dt=dt * s, kind=kind)])
+        h.set_T(0, T0)
+        h.step(1)
+        G_ = dt * N * N / 3.0 * (np.max(Us) ** 0.75 if okind == "t3" else 1.0)
+        assert np.max(np.abs(h.T(0) - T)) / np.max(T) < 4 * 2.2e-16 * (1 + 4 * G_)
+        assert np.max(np.abs(h.Ustar(0) - Us)) / np.max(Us) < 1e-13
+        h.close()
