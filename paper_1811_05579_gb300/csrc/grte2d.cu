@@ -1551,8 +1551,7 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
             alloc2(h, &D.newton_its, nc) && alloc2(h, &D.acU, nc) && alloc2(h, &D.status, 1) &&
             alloc2(h, &D.wsc, nc) && alloc2(h, &D.iwsc, nc) && alloc2(h, &D.gd, K * nc) && alloc2(h, &D.gdi, K * nc) && alloc2(h, &D.pdi, nc) &&
             alloc2(h, &h->V, K * nv) && alloc2(h, &h->phi, K * nc) && alloc2(h, &h->GU, K * nc) &&
-            alloc2(h, &h->Es, K * nc) && alloc2(h, &h->b, nz) && alloc2(h, &h->x, nz) && alloc2(h, &h->Kr, nz) &&
-            alloc2(h, &h->Kt, nz) &&
+            alloc2(h, &h->Es, K * nc) && alloc2(h, &h->b, nz) && alloc2(h, &h->x, nz) &&
             // also the scratch of K nv vertex values between solves (2 x 2 cells, m = 1: the larger)
             alloc2(h, &h->Kbasis, std::max((int64_t)(h->m + 1) * basis_ld(nz), K * nv)) &&
             alloc2(h, &h->part, (int64_t)kAxpyBlocks * (kMaxRestart2 + 1)) && alloc2(h, &h->dots, kMaxRestart2 + 1) &&
@@ -1565,6 +1564,11 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
   CK2(op_attrs());
   if (h->opt.prec2d & ~(GRTE_PREC2D_MULTIGRID | GRTE_PREC2D_CORR_MG))
     return fail2(h, GRTE_EINVAL, "prec2d: a set of GRTE_PREC2D_MULTIGRID and GRTE_PREC2D_CORR_MG");
+  // M z before a multigrid preconditioner (the per-cell one is applied in the operator pass), the
+  // Schur multigrid's probe and elimination vector
+  if (h->opt.prec2d != 0 && !alloc2(h, &h->Kr, nz)) return fail2(h, GRTE_ENOMEM, "cudaMalloc multigrid vectors");
+  if ((h->opt.prec2d & GRTE_PREC2D_MULTIGRID) && !alloc2(h, &h->Kt, nz))
+    return fail2(h, GRTE_ENOMEM, "cudaMalloc multigrid vectors");
   if (h->opt.prec2d & GRTE_PREC2D_CORR_MG) {
     // levels of 2x2 aggregates down to lines of <= 2 cells in both axes
     mp::PLevel L{};
@@ -1613,7 +1617,8 @@ grte_status grte2d_create(const grte_instance2d* p, const grte_options* opt, grt
                alloc2(h, &h->kc32, nc) && alloc2(h, &h->A32, nc) && alloc2(h, &h->alpha32, nc) &&
                alloc2(h, &h->dv32, nv) && alloc2(h, &h->gd32, K * nc) && alloc2(h, &h->gdi32, K * nc) &&
                alloc2(h, &h->pdi32, nc) && alloc2(h, &h->wsc32, nc) && alloc2(h, &h->iwsc32, nc) &&
-               alloc2(h, &h->V32, (int64_t)(h->m + 1) * basis_ld(nz)) && alloc2(h, &h->Kr32, nz);
+               alloc2(h, &h->V32, (int64_t)(h->m + 1) * basis_ld(nz)) &&
+               (!(h->opt.prec2d & GRTE_PREC2D_CORR_MG) || alloc2(h, &h->Kr32, nz));
     if (!okf) return fail2(h, GRTE_ENOMEM, "cudaMalloc binary32 buffers");
     std::vector<float> f(K);
     for (int64_t k = 0; k < K; ++k) f[k] = (float)h->hmu[k];
