@@ -38,21 +38,20 @@ HOM_FLOPS_PER_ELEM = 31
 # factor values read (1/den, a, c-hat, c-check, a-check) and the flux contribution
 # written; the line's unknowns stay in shared memory.
 LINE_BYTES_PER_ELEM_F32 = 5 * 4 + 4
-# Bytes a Krylov-kernel launch (k_gmres, one cluster of 8 CTAs per instance) must move
-# per cell: the e/o flux parts of all M angles of the pass before it (bulk type) and
+# Bytes a Krylov-kernel launch (k_gmres, one cluster of 8 or 16 CTAs per instance) must move
+# per cell: what the pass before it left of all M angles (flux parts, in FP64 differences of e) and
 # four double per-cell vectors (direction or iterate in, result out, two basis reads).
 GMRES_BYTES_PER_CELL = lambda M, es: M * es + 4 * 8
 # DRAM bytes per k_gmres<ARNOLDI> launch measured by ncu --set full (mean of two
 # launches, cold cache) on the 1D slab workload in mixed precision.  The kernel has
-# changed since (restart decision read before the CTAs' barriers); until the counters
-# are taken again the line reports traffic as null and gives this figure as context.
+# changed since (loads ahead of their chains, fewer barriers, one CTA for small grids); until
+# the counters are taken again the line reports traffic as null and gives this figure as context.
 GMRES_TRAFFIC_SLAB6_MIXED_EARLIER = 13.19e6
-# DRAM bytes per k_gmres launch on the 1D slab workload in FP64, the mean over six
-# consecutive launches of all modes (restart 18.4 MB, Arnoldi 3.8 and 3.7 MB, update 3.0
-# and 1.0 MB, one launch whose instances had all stopped 0.07 MB; ncu dram__bytes_read.sum
-# + dram__bytes_write.sum, profiles/ncu_gmres_fp64_slab6.md), taken with the kernel as it
-# stands
-GMRES_DRAM_BYTES_SLAB6_FP64 = 5.00e6
+# DRAM bytes per k_gmres launch on the 1D slab workload in FP64, the mean over all 50 launches of
+# five steps (29 Arnoldi steps 12.3 MB, 9 restarts 16.5 MB, 3 first restarts 21.4 MB, 9 updates 3.6
+# MB; ncu dram__bytes_read.sum + dram__bytes_write.sum, profiles/ncu_gmres_fp64_slab6.md), taken
+# with the kernel as it stands (clusters of sixteen CTAs)
+GMRES_DRAM_BYTES_SLAB6_FP64 = 12.00e6
 # Per-cell bytes the fused prediction solve must move besides the state: the binary64
 # inputs it reads once (T^n, U^n, rho^n and the 16 coefficient arrays of the cell) and
 # the outputs rho* and F* (20 x 8 B).
@@ -60,7 +59,7 @@ FUSED_BYTES_PER_CELL = 160
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_pred_fused launch on one 8192-cell,
 # 64-direction slab run (ncu --set full; profiles/ncu_pred_fused_slab1.md), taken with the
 # kernel as it stands; a slab launch carries one such instance per run
-FUSED_DRAM_BYTES_SLAB_INSTANCE = 4.137216e6
+FUSED_DRAM_BYTES_SLAB_INSTANCE = 4.144896e6
 
 
 def job_throughput(updates_per_step, steps, t_ms, world, dist=None, device="cuda"):
@@ -162,7 +161,7 @@ def roofline_of(prof, runs, prec, hbm_peak, workload):
                 "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)",
                 "traffic": GMRES_DRAM_BYTES_SLAB6_FP64 if (workload == "slab6" and prec == G.FP64) else None,
-                "traffic_source": "ncu dram bytes, mean of six launches of all modes",
+                "traffic_source": "ncu dram bytes, mean of the 50 launches of five steps",
                 "traffic_before_last_kernel_change": earlier,
                 "avg_launch_us": avg_s * 1e6, "launches": dom_n, "bytes_per_cell": GMRES_BYTES_PER_CELL(M, es),
                 "bytes_model": "achieved and frac from the byte model: M x %d B flux parts + 4 x 8 B per cell" % es}

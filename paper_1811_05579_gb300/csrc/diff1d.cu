@@ -62,11 +62,12 @@ __device__ __forceinline__ double d_pow34(double u) {
 }
 
 // The positive root of t^4 + beta t = R (beta, R > 0): Newton from
-// T_hi = min(R^{1/4}, R/beta), monotone (convex increasing left side).  Within the binary32
-// range five steps there reach its rounding (T_hi is at most 2^{1/4} above the root) and two
-// binary64 steps, their slope's reciprocal in binary32, finish: the errors go
-// 2e-7 -> 6e-14 -> rounding.  Elsewhere all steps are binary64, until t stops decreasing;
-// false if maxit steps do not suffice.
+// T_hi = min(R^{1/4}, R/beta), monotone (convex increasing left side).  T_hi is at most 1.381
+// times the root (at beta = R^{3/4}, t^4 + t = 1), from where exact Newton errors go 0.10,
+// 9.3e-3, 7.8e-5, 5.5e-9: within the binary32 range five steps there reach its rounding, and two
+// binary64 steps, their slope's reciprocal in binary32, finish: 2e-7 -> 6e-14 -> rounding (worst
+// 4.4e-16 over 2e6 arguments of the whole range).  Elsewhere all steps are binary64, until t
+// stops decreasing; false if maxit steps do not suffice.
 __device__ __forceinline__ bool d_root(double beta, double R, int maxit, double& t) {
   const float rf = (float)R, bf = (float)beta;
   if (rf > 1e-20f && rf < 1e20f && bf > 1e-20f && bf < 1e20f) {

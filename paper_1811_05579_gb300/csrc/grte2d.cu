@@ -1038,7 +1038,10 @@ static cudaError_t op_attr(int bytes) {
   if (e == cudaSuccess) e = set((const void*)k2_op<S, PRED, PREC, RES, 8, 4, 10>);
   return e;
 }
-// The operator kernels' shared-memory limit (kMaxPairs binary64 pairs need 166 KB).
+// The operator kernels' shared-memory limit (kMaxPairs binary64 pairs need 141 KB, 32 x 8 tiles).
+static_assert(op_smem<double>(kMaxPairs, 32, 8, 1, true) == 143848 && op_smem<double>(kMaxPairs, 32, 4, 4, true) < 143848 &&
+                  op_smem<double>(kMaxPairs, 8, 4, 10, true) < 143848,
+              "every tiling fits the 227 KB of a CTA");
 static cudaError_t op_attrs() {
   int dev = 0, bytes = 0;
   cudaError_t e = cudaGetDevice(&dev);

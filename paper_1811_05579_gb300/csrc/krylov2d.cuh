@@ -311,8 +311,9 @@ __device__ __forceinline__ bool last_block(unsigned* count) {
   return last;
 }
 
-// Block sums of C values per thread (C a power of two), in binary64, to
-// part[(i0 + t) * gridDim.x + block] for t < nv.  A warp leaves each lane one value's sum by
+// Block sums of C values per thread (C a power of two), within a warp in the vectors' type and
+// across warps in binary64, to part[(i0 + t) * gridDim.x + block] for t < nv.  A warp leaves each
+// lane one value's sum by
 // halving the values it holds with every exchange (C - 1 + 5 - log2 C additions instead of
 // 5 C: a binary64 warp addition holds its sub-partition's pipe for many cycles).
 template <typename S, int C>
@@ -501,7 +502,8 @@ __device__ __forceinline__ void krylov_column(KState* ks, int j, double hn2, KSt
 
 // w -= sum_{i <= j} coef_i V_i and |w|^2.  Pass 1 decides whether w has to be orthogonalised
 // again (binary64: when little of it is left, so that the rounding of the first pass weighs:
-// |w|^2 <= 1e-2 |w before|^2; binary32 cycles, which only have to gain 1e5 and whose restarts
+// |w|^2 <= 1e-2 |w before|^2, which takes the same steps to the same errors as a second pass
+// always, on 192^2 and 61 x 47 cells 1.21x and 1.18x as fast; binary32 cycles, which only have to gain 1e5 and whose restarts
 // are binary64, never); the last pass finishes the column.
 // C: vectors of a chunk, loaded together (past the last one it is loaded again, with a zero
 // coefficient); U groups of 16 bytes per thread and turn.
