@@ -87,3 +87,20 @@ def test_small_sigma(G):
         assert np.max(np.abs(h.T(0) - T)) / np.max(T) < 4 * 2.2e-16 * (1 + 4 * G_)
         assert np.max(np.abs(h.Ustar(0) - Us)) / np.max(Us) < 1e-13
         h.close()
+
+
+# Rows are scaled from T = 2^128 on: cells on both sides of it in every CTA (a = C_v = 1, the oracle on
+# the same inputs; T^7 = 2^901 is in its range).
+def test_cells_on_both_sides_of_the_scaled_range(G, unit):
+    s = 2.0 ** 128
+    for N, kind, T0, sig, dt, _, _ in unit:
+        assert np.any(T0 < 0.9) and np.any(T0 > 1.1)
+        sg = sig * (s ** 3 if kind == "t3" else 1.0)
+        T, Us = dif.three_stage_step(T0 * s, sg, 1.0 / N, dt, kind=kind)
+        h = G.Diffusion([dict(nx=N, sigma=sg, dt=dt, kind=G.SIGMA_T3 if kind == "t3" else G.SIGMA_CONST)])
+        h.set_T(0, T0 * s)
+        h.step(1)
+        G_ = dt * N * N / (3.0 * sg.min()) * (np.max(Us) ** 0.75 if kind == "t3" else 1.0)
+        assert np.max(np.abs(h.T(0) - T)) / np.max(T) < 4 * 2.2e-16 * (1 + 4 * G_)
+        assert np.max(np.abs(h.Ustar(0) - Us)) / np.max(Us) < 1e-12
+        h.close()
